@@ -54,7 +54,7 @@ __global__ void reduce_eta_kernel(const double* __restrict__ partials, int np, S
     const double sum = sh[0];
     double eta;
     if (t0 > 0.0) eta = sqrt(sum / t0);
-    else eta = (sum > 0.0) ? INFINITY : 0.0;
+    else eta = (t0 == 0.0 && sum == 0.0) ? 0.0 : INFINITY;  // (a NaN is neither)
     const int it = st->it + 1;
     st->it = it;
     const double prev = st->eta;
@@ -100,7 +100,7 @@ __global__ void reduce_crit_kernel(const double* __restrict__ partials, const do
     st->restart = 0;
     const double* t = st->T0;
     const double t0 = t[0] * t[0] + t[1] * t[1] + t[2] * t[2] + 2.0 * (t[3] * t[3] + t[4] * t[4] + t[5] * t[5]);
-    const double eta = t0 > 0.0 ? sqrt(s / t0) : (s > 0.0 ? INFINITY : 0.0);
+    const double eta = t0 > 0.0 ? sqrt(s / t0) : (t0 == 0.0 && s == 0.0 ? 0.0 : INFINITY);
     const int it = st->it + 1;
     st->it = it;
     const double prev = st->eta;
@@ -536,7 +536,7 @@ struct gfp_grid_s {
   int phase_gen = 0;          // incremented by gfp_set_phases and gfp_set_tiles (batch graphs bake both in)
   double* eps = nullptr;
   double2* spec = nullptr;
-  double2* tw64[3] = {nullptr, nullptr, nullptr};
+  fxw* tw64[3] = {nullptr, nullptr, nullptr};
   double* tabA[3] = {nullptr, nullptr, nullptr};
   double* tabB[3] = {nullptr, nullptr, nullptr};
   int table_op = -1;
@@ -696,6 +696,40 @@ LaunchCfg make_cfg(const Dims& d, int eb) {
   return c;
 }
 
+// e^{-2 pi i j / n} as a fixed-point table entry.  The angle is folded to u / n eighths of a turn, 0 <= u <= n, so that the
+// table has the circle's symmetries and its zeros and ones exactly; cosine and sine there are their power series
+// in 63-bit fractions (an error of a few 2^-63, the same on every host).
+fxw fx_twiddle_entry(int n, int j) {
+  typedef unsigned __int128 u128;
+  const unsigned long long one = 1ull << 63, quarter_pi = 0x6487ed5110b4611aull;  // pi/4 2^63
+  const int oct = (int)((8LL * j) / n) & 7;
+  const long long rem = (8LL * j) % n, u = (oct & 1) ? n - rem : rem;
+  const unsigned long long x = (unsigned long long)((u128)quarter_pi * (unsigned long long)u / (unsigned long long)n);
+  auto mul = [](unsigned long long a, unsigned long long b) { return (unsigned long long)(((u128)a * b) >> 63); };
+  const unsigned long long x2 = mul(x, x);
+  unsigned long long c = one, s = one;
+  for (int k = 12; k >= 1; --k) {
+    c = one - mul(x2, c) / (unsigned long long)((2 * k - 1) * (2 * k));
+    s = one - mul(x2, s) / (unsigned long long)((2 * k) * (2 * k + 1));
+  }
+  s = mul(x, s);
+  long long cq = (long long)((c + 1) >> 1), sq = (long long)((s + 1) >> 1);  // Q62
+  const bool swap = oct == 1 || oct == 2 || oct == 5 || oct == 6;
+  long long re = swap ? sq : cq, im = swap ? cq : sq;
+  if (oct >= 2 && oct <= 5) re = -re;
+  if (oct < 4) im = -im;  // e^{-i theta}
+  auto split = [](long long v, int& h, int& l) {
+    long long lo = (long long)(int)(unsigned)(v & 0xffffffffll);
+    if (lo == -2147483648LL) lo = -2147483647LL;  // its negative has to be an int
+    h = (int)((v - lo + 1) >> 32);
+    l = (int)lo;
+  };
+  fxw w;
+  split(re, w.xh, w.xl);
+  split(im, w.yh, w.yl);
+  return w;
+}
+
 // cuTensorMapEncodeTiled from the driver (looked up once; null if unavailable).
 PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
   static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
@@ -853,6 +887,11 @@ int ensure_hist(gfp_grid g, int cap) {
   return GFP_OK;
 }
 
+// F and HC average the Green operator over Hermitian partners on the Nyquist planes, which only even axes have.
+int nyquist_average(int op, const Dims& d) {
+  return (op == OP_F || op == OP_HC) && (d.n1 % 2 == 0 || d.n2 % 2 == 0 || d.n3 % 2 == 0) ? 1 : 0;
+}
+
 // x-pass parameters of the FP64 passes: the eigenstrain while one is set
 PolarParams fp64_xparams(gfp_grid g) {
   PolarParams pp;
@@ -869,7 +908,7 @@ void one_iteration64(gfp_grid g, const GammaParams<double>& gp, int have_delta, 
   g->launches += 5;
   const PolarParams pp = fp64_xparams(g);
   Passes<double>::pass_x(g->stream, lc, g->spec, g->eps, g->lam, g->mu, g->tw64[0], lc.plan[0], d,
-                         have_delta ? PX_DELTA : 0, nullptr, nullptr, g->st, &pp);
+                         have_delta ? PX_DELTA : 0, g->st, &pp);
   Passes<double>::pass_y(g->stream, lc, false, g->spec, g->tw64[1], lc.plan[1], d, g->st);
   Passes<double>::pass_z(g->stream, lc, g->spec, g->tw64[2], lc.plan[2], d, gp, g->partials, g->st, PZ_GAMMA,
                          nullptr);
@@ -895,7 +934,7 @@ int solve_fp64(gfp_grid g, const gfp_scheme* sc, const double E[6], double tol, 
   gp.c_mu = 1.0 / (2.0 * g->mu_h);
   gp.c_lm = (g->lam_h + g->mu_h) / (g->mu_h * (g->lam_h + 2.0 * g->mu_h));
   gp.invN = 1.0 / (double)g->d.N;
-  gp.nyq_avg = (sc->op == OP_F || sc->op == OP_HC) ? 1 : 0;
+  gp.nyq_avg = nyquist_average(sc->op, g->d);
   gp.half_shift = 0;
   gp.dgo = nullptr;
   // the paper's increment rule: the previous iteration's T kt per point and the criterion partials
@@ -1012,10 +1051,12 @@ int ensure_mixed(gfp_grid g) {
     GFP_CU(cudaMalloc(&g->tw32[r], sizeof(float2) * ns[r]));
     GFP_CU(cudaMalloc(&g->tabA32[r], sizeof(float) * ns[r]));
     GFP_CU(cudaMalloc(&g->tabB32[r], sizeof(float) * ns[r]));
-    std::vector<double2> tw(ns[r]);
-    GFP_CU(cudaMemcpy(tw.data(), g->tw64[r], sizeof(double2) * ns[r], cudaMemcpyDeviceToHost));
     std::vector<float2> twf(ns[r]);
-    for (int j = 0; j < ns[r]; ++j) { twf[j].x = (float)tw[j].x; twf[j].y = (float)tw[j].y; }
+    for (int j = 0; j < ns[r]; ++j) {  // w_n^j = e^{-2 pi i j / n}
+      const double a = -2.0 * 3.14159265358979323846 * (double)j / (double)ns[r];
+      twf[j].x = (float)std::cos(a);
+      twf[j].y = (float)std::sin(a);
+    }
     GFP_CU(cudaMemcpy(g->tw32[r], twf.data(), sizeof(float2) * ns[r], cudaMemcpyHostToDevice));
   }
   GFP_CU(cudaMalloc(&g->st_in, sizeof(SolveState)));
@@ -1052,7 +1093,7 @@ GammaParams<R> gamma_params(gfp_grid g, int op, const R* const* A, const R* cons
   gp.c_mu = (R)(1.0 / (2.0 * g->mu_h));
   gp.c_lm = (R)((g->lam_h + g->mu_h) / (g->mu_h * (g->lam_h + 2.0 * g->mu_h)));
   gp.invN = (R)(1.0 / (double)g->d.N);
-  gp.nyq_avg = (op == OP_F || op == OP_HC) ? 1 : 0;
+  gp.nyq_avg = nyquist_average(op, g->d);
   gp.half_shift = (op == OP_AFB_R) ? 1 : 0;
   gp.dgo = nullptr;
   return gp;
@@ -1117,8 +1158,7 @@ void inner_iteration32(gfp_grid g, const GammaParams<float>& gp, int flags) {
   const Dims& d = g->d;
   g->launches += 5;
   float2* spec32 = reinterpret_cast<float2*>(g->spec);
-  Passes<float>::pass_x(g->stream, g->lc32, spec32, g->eps32, g->lam32, g->mu32, g->tw32[0], g->lc32.plan[0], d, flags,
-                        nullptr, nullptr, g->st_in);
+  Passes<float>::pass_x(g->stream, g->lc32, spec32, g->eps32, g->lam32, g->mu32, g->tw32[0], g->lc32.plan[0], d, flags, g->st_in);
   Passes<float>::pass_y(g->stream, g->lc32, false, spec32, g->tw32[1], g->lc32.plan[1], d, g->st_in);
   Passes<float>::pass_z(g->stream, g->lc32, spec32, g->tw32[2], g->lc32.plan[2], d, gp, g->partials, g->st_in, PZ_INNER,
                         g->vsrc);
@@ -1355,7 +1395,7 @@ int solve_dgo(gfp_grid g, const gfp_scheme* sc, const double E[6], double tol, i
     for (int b = 0; b < nb; ++b) {
       const int j = launched + b;
       Passes<double>::pass_x(g->stream, g->lc64, g->spec, g->eps, g->lam, g->mu, g->tw64[0], g->lc64.plan[0], d,
-                             (stress_form ? PX_DRES : PX_POLAR) | (j > 0 ? PX_DELTA : 0), nullptr, nullptr, g->st,
+                             (stress_form ? PX_DRES : PX_POLAR) | (j > 0 ? PX_DELTA : 0), g->st,
                              &pp);
       if (j > 0) reduce_dgo_kernel<<<1, 256, 0, g->stream>>>(g->xpart, np, enorm, g->st, g->hist, g->hist_cap);
       g->launches += j > 0 ? 5 : 4;
@@ -1519,7 +1559,7 @@ int gfp_create_grid(int n1, int n2, int n3, double h, void* cuda_stream, gfp_gri
   A((void**)&g->eps, sizeof(double) * 6 * d.N);
   A((void**)&g->spec, sizeof(double2) * 6 * d.S);
   for (int r = 0; r < 3; ++r) {
-    A((void**)&g->tw64[r], sizeof(double2) * ns[r]);
+    A((void**)&g->tw64[r], sizeof(fxw) * ns[r]);
     A((void**)&g->tabA[r], sizeof(double) * ns[r]);
     A((void**)&g->tabB[r], sizeof(double) * ns[r]);
   }
@@ -1530,16 +1570,10 @@ int gfp_create_grid(int n1, int n2, int n3, double h, void* cuda_stream, gfp_gri
   A((void**)&g->bad, sizeof(unsigned long long));
   if (e == cudaSuccess) e = cudaMallocHost((void**)&g->st_host, sizeof(SolveState));
   if (e != cudaSuccess) { note_error(e, __LINE__); free_grid(g); return cuda_status(e); }
-  // twiddles w_n^j = e^{-2 pi i j / n}
-  const double pi = 3.14159265358979323846;
   for (int r = 0; r < 3; ++r) {
-    std::vector<double2> tw(ns[r]);
-    for (int j = 0; j < ns[r]; ++j) {
-      const double a = -2.0 * pi * (double)j / (double)ns[r];
-      tw[j].x = std::cos(a);
-      tw[j].y = std::sin(a);
-    }
-    e = cudaMemcpy(g->tw64[r], tw.data(), sizeof(double2) * ns[r], cudaMemcpyHostToDevice);
+    std::vector<fxw> tw(ns[r]);
+    for (int j = 0; j < ns[r]; ++j) tw[j] = fx_twiddle_entry(ns[r], j);
+    e = cudaMemcpy(g->tw64[r], tw.data(), sizeof(fxw) * ns[r], cudaMemcpyHostToDevice);
     if (e != cudaSuccess) { free_grid(g); return cuda_status(e); }
   }
   e = cudaMemsetAsync(g->spec, 0, sizeof(double2) * 6 * d.S, g->stream);
@@ -1654,14 +1688,13 @@ int gfp_get_displacement(gfp_grid g, const gfp_scheme* sc, double* dst, int wher
   *g->st_host = s0;
   GFP_CU(cudaMemcpyAsync(g->st, g->st_host, sizeof(SolveState), cudaMemcpyHostToDevice, g->stream));
   // forward transform of eps - E_bar, u^ per mode, inverse transform of its 3 components
-  Passes<double>::pass_x(g->stream, g->lc64, g->spec, g->eps, g->lam, g->mu, g->tw64[0], g->lc64.plan[0], d, PX_STRAIN,
-                         nullptr, nullptr, g->st, &pp);
+  Passes<double>::pass_x(g->stream, g->lc64, g->spec, g->eps, g->lam, g->mu, g->tw64[0], g->lc64.plan[0], d, PX_STRAIN, g->st, &pp);
   Passes<double>::pass_y(g->stream, g->lc64, false, g->spec, g->tw64[1], g->lc64.plan[1], d, g->st);
   Passes<double>::pass_z(g->stream, g->lc64, g->spec, g->tw64[2], g->lc64.plan[2], d, gp, g->partials, g->st, PZ_DISP,
                          nullptr);
   Passes<double>::pass_y(g->stream, g->lc64, true, g->spec, g->tw64[1], g->lc64.plan[1], d, g->st);
   Passes<double>::pass_x(g->stream, g->lc64, g->spec, out, g->lam, g->mu, g->tw64[0], g->lc64.plan[0], d,
-                         PX_DELTA | PX_OUTPUT, nullptr, nullptr, g->st, &pp);
+                         PX_DELTA | PX_OUTPUT, g->st, &pp);
   GFP_CU(cudaGetLastError());
   if (where == 0) GFP_CU(cudaMemcpyAsync(dst, out, bytes, cudaMemcpyDeviceToHost, g->stream));
   GFP_CU(cudaStreamSynchronize(g->stream));
@@ -1795,10 +1828,9 @@ int gfp_time_passes(gfp_grid g, const gfp_scheme* sc, int iters, double pass_ms[
     GFP_CU(cudaEventRecord(ev[0], g->stream));
     if (mixed)
       Passes<float>::pass_x(g->stream, g->lc32, spec32, g->eps32, g->lam32, g->mu32, g->tw32[0], g->lc32.plan[0], d,
-                            PX_DELTA, nullptr, nullptr, g->st_in);
+                            PX_DELTA, g->st_in);
     else
-      Passes<double>::pass_x(g->stream, g->lc64, g->spec, g->eps, g->lam, g->mu, g->tw64[0], g->lc64.plan[0], d, PX_DELTA,
-                             nullptr, nullptr, g->st);
+      Passes<double>::pass_x(g->stream, g->lc64, g->spec, g->eps, g->lam, g->mu, g->tw64[0], g->lc64.plan[0], d, PX_DELTA, g->st);
     GFP_CU(cudaEventRecord(ev[1], g->stream));
     if (mixed) Passes<float>::pass_y(g->stream, g->lc32, false, spec32, g->tw32[1], g->lc32.plan[1], d, g->st_in);
     else Passes<double>::pass_y(g->stream, g->lc64, false, g->spec, g->tw64[1], g->lc64.plan[1], d, g->st);
@@ -1884,7 +1916,7 @@ int gfp_solve_noalloc(int n1, int n2, int n3, double h, const double* lambda, co
   size_t off = 0;
   const size_t o_spec = off; off = align256(off + sizeof(double2) * 6 * (size_t)d.S);
   size_t o_tw[3], o_A[3], o_B[3];
-  for (int r = 0; r < 3; ++r) { o_tw[r] = off; off = align256(off + sizeof(double2) * ns[r]); }
+  for (int r = 0; r < 3; ++r) { o_tw[r] = off; off = align256(off + sizeof(fxw) * ns[r]); }
   for (int r = 0; r < 3; ++r) { o_A[r] = off; off = align256(off + sizeof(double) * ns[r]); }
   for (int r = 0; r < 3; ++r) { o_B[r] = off; off = align256(off + sizeof(double) * ns[r]); }
   const size_t o_part = off; off = align256(off + sizeof(double) * (size_t)lc.z_blocks);
@@ -1907,27 +1939,24 @@ int gfp_solve_noalloc(int n1, int n2, int n3, double h, const double* lambda, co
   double2* spec = reinterpret_cast<double2*>(sb + o_spec);
   double* partials = reinterpret_cast<double*>(sb + o_part);
   SolveState* st = reinterpret_cast<SolveState*>(sb + o_st);
-  double2* tw[3];
+  fxw* tw[3];
   GammaParams<double> gp;
   // twiddles and wave-vector tables, staged through a small host buffer
-  const double pi = 3.14159265358979323846;
   for (int r = 0; r < 3; ++r) {
-    tw[r] = reinterpret_cast<double2*>(sb + o_tw[r]);
+    tw[r] = reinterpret_cast<fxw*>(sb + o_tw[r]);
     double* A = reinterpret_cast<double*>(sb + o_A[r]);
     double* B = reinterpret_cast<double*>(sb + o_B[r]);
     gp.A[r] = A;
     gp.B[r] = B;
     for (int j0 = 0; j0 < ns[r]; j0 += 64) {
-      double2 t64[64];
+      fxw t64[64];
       double a64[64], b64[64];
       const int cnt = std::min(64, ns[r] - j0);
       for (int j = 0; j < cnt; ++j) {
-        const double ang = -2.0 * pi * (double)(j0 + j) / (double)ns[r];
-        t64[j].x = std::cos(ang);
-        t64[j].y = std::sin(ang);
+        t64[j] = fx_twiddle_entry(ns[r], j0 + j);
         table_entry(sc->op, ns[r], j0 + j, h, &a64[j], &b64[j]);
       }
-      GFP_CU(cudaMemcpyAsync(tw[r] + j0, t64, sizeof(double2) * cnt, cudaMemcpyHostToDevice, stream));
+      GFP_CU(cudaMemcpyAsync(tw[r] + j0, t64, sizeof(fxw) * cnt, cudaMemcpyHostToDevice, stream));
       GFP_CU(cudaMemcpyAsync(A + j0, a64, sizeof(double) * cnt, cudaMemcpyHostToDevice, stream));
       GFP_CU(cudaMemcpyAsync(B + j0, b64, sizeof(double) * cnt, cudaMemcpyHostToDevice, stream));
       GFP_CU(cudaStreamSynchronize(stream));
@@ -1964,7 +1993,7 @@ int gfp_solve_noalloc(int n1, int n2, int n3, double h, const double* lambda, co
   gp.c_mu = 1.0 / (2.0 * mu_h);
   gp.c_lm = (lam_h + mu_h) / (mu_h * (lam_h + 2.0 * mu_h));
   gp.invN = 1.0 / (double)d.N;
-  gp.nyq_avg = (sc->op == OP_F || sc->op == OP_HC) ? 1 : 0;
+  gp.nyq_avg = nyquist_average(sc->op, d);
   gp.half_shift = 0;
   gp.dgo = nullptr;
   // the shared scratch keeps the previous call's contents: clear the spectrum, reset the state
@@ -1984,7 +2013,7 @@ int gfp_solve_noalloc(int n1, int n2, int n3, double h, const double* lambda, co
     const int nb = std::min(chunk, maxit - launched);
     for (int b = 0; b < nb; ++b) {
       const int flags = (launched + b) > 0 ? PX_DELTA : 0;
-      Passes<double>::pass_x(stream, lc, spec, eps, lambda, mu, tw[0], lc.plan[0], d, flags, nullptr, nullptr, st);
+      Passes<double>::pass_x(stream, lc, spec, eps, lambda, mu, tw[0], lc.plan[0], d, flags, st);
       Passes<double>::pass_y(stream, lc, false, spec, tw[1], lc.plan[1], d, st);
       Passes<double>::pass_z(stream, lc, spec, tw[2], lc.plan[2], d, gp, partials, st, PZ_GAMMA, nullptr);
       launch_reduce_eta(stream, partials, lc.z_blocks, st, nullptr, 0);
@@ -2037,11 +2066,9 @@ int gfp_tune(gfp_grid g, const gfp_scheme* sc, int iters, int tiles_out[3]) {
     for (int i = 0; i < iters; ++i) {
       if (pass == 0) {
         if (mixed)
-          Passes<float>::pass_x(g->stream, c, spec32, g->eps32, g->lam32, g->mu32, g->tw32[0], c.plan[0], d, PX_DELTA,
-                                nullptr, nullptr, g->st_in);
+          Passes<float>::pass_x(g->stream, c, spec32, g->eps32, g->lam32, g->mu32, g->tw32[0], c.plan[0], d, PX_DELTA, g->st_in);
         else
-          Passes<double>::pass_x(g->stream, c, g->spec, g->eps, g->lam, g->mu, g->tw64[0], c.plan[0], d, PX_DELTA,
-                                 nullptr, nullptr, g->st);
+          Passes<double>::pass_x(g->stream, c, g->spec, g->eps, g->lam, g->mu, g->tw64[0], c.plan[0], d, PX_DELTA, g->st);
       } else if (pass == 1) {
         if (mixed) Passes<float>::pass_y(g->stream, c, false, spec32, g->tw32[1], c.plan[1], d, g->st_in);
         else Passes<double>::pass_y(g->stream, c, false, g->spec, g->tw64[1], c.plan[1], d, g->st);
@@ -2260,8 +2287,7 @@ void slot_window(BatchSlot& s, int op, const GammaParams<float>& gp32, const Bat
   batch_arm_kernel<<<1, 32, 0, st>>>(s.st, s.st_in, s.acc, ctl, kInnerReduction, window);
   float2* spec32 = reinterpret_cast<float2*>(s.spec);
   for (int k = 0; k < window; ++k) {
-    Passes<float>::pass_x(st, s.lc32, spec32, s.eps32, g->lam32, g->mu32, g->tw32[0], s.lc32.plan[0], d, PX_DELTA,
-                          nullptr, nullptr, s.st_in);
+    Passes<float>::pass_x(st, s.lc32, spec32, s.eps32, g->lam32, g->mu32, g->tw32[0], s.lc32.plan[0], d, PX_DELTA, s.st_in);
     Passes<float>::pass_y(st, s.lc32, false, spec32, g->tw32[1], s.lc32.plan[1], d, s.st_in);
     Passes<float>::pass_z(st, s.lc32, spec32, g->tw32[2], s.lc32.plan[2], d, gp32, s.partials, s.st_in, PZ_INNER, s.vsrc);
     launch_reduce_eta(st, s.partials, s.lc32.z_blocks, s.st_in, nullptr, 0);

@@ -506,14 +506,13 @@ __global__ void __launch_bounds__(24 * CPlan<N>::T, 2) pass_z_c2_kernel(typename
 
 // ------------------------------------------------------------------------------------------------
 // pass_x: CTA = `lines` x1-lines (consecutive i2 at fixed i3) x 3 component pairs; thread = (pair
-// line, t).  Same flags and correction as the generic kernel.
+// line, t).  Same flags as the generic kernel.
 // ------------------------------------------------------------------------------------------------
 template <typename R, int N>
 __global__ void __launch_bounds__(512) pass_x_c_kernel(typename C<R>::T* __restrict__ spec, R* __restrict__ eps,
                                                        const R* __restrict__ lam, const R* __restrict__ mu,
                                                        const typename C<R>::T* __restrict__ tw, Dims d, int lines,
-                                                       int flags, const float* __restrict__ corr,
-                                                       const double* __restrict__ corr_mean, PolarParams pp,
+                                                       int flags, PolarParams pp,
                                                        const SolveState* __restrict__ st) {
   typedef typename C<R>::T T;
   typedef CPlan<N> P;
@@ -569,11 +568,6 @@ __global__ void __launch_bounds__(512) pass_x_c_kernel(typename C<R>::T* __restr
   __syncthreads();
   const bool polar = (flags & PX_POLAR) != 0;
   double dacc = 0.0;
-  double cm[6];
-  if (corr) {
-#pragma unroll
-    for (int c = 0; c < 6; ++c) cm[c] = corr_mean[c];
-  }
   // XU voxels per step, all their loads issued before any store: a plain loop waits one DRAM latency
   // per voxel, since its strain loads are ordered after the previous voxel's stores to the same array
   // (FP32: 2 voxels at 64 registers; FP64 keeps 1, its registers are already at the launch bound)
@@ -623,11 +617,7 @@ __global__ void __launch_bounds__(512) pass_x_c_kernel(typename C<R>::T* __restr
         for (int c = 0; c < 6; ++c) e[c] += dd[c];
       }
     }
-    if (corr) {
-#pragma unroll
-      for (int c = 0; c < 6; ++c) e[c] += (R)((double)corr[c * d.N + vv] - cm[c]);
-    }
-    if (have_delta || zero || corr) {
+    if (have_delta || zero) {
 #pragma unroll
       for (int c = 0; c < 6; ++c) eps[c * d.N + vv] = e[c];
     }
@@ -709,8 +699,7 @@ template <typename R, int N>
 __global__ void __launch_bounds__(512) pass_x_a_kernel(typename C<R>::T* __restrict__ spec, R* __restrict__ eps,
                                                        const R* __restrict__ lam, const R* __restrict__ mu,
                                                        const typename C<R>::T* __restrict__ tw, Dims d, int lines,
-                                                       int flags, const float* __restrict__ corr,
-                                                       const double* __restrict__ corr_mean,
+                                                       int flags,
                                                        const SolveState* __restrict__ st) {
   typedef typename C<R>::T T;
   typedef CPlan<N> P;
@@ -785,11 +774,6 @@ __global__ void __launch_bounds__(512) pass_x_a_kernel(typename C<R>::T* __restr
       for (int r = 0; r < RL; ++r) sl[cout_idx<N, P::NST - 1>(t, b, r)] = v[b * RL + r];
   }
   __syncthreads();
-  double cm[6];
-  if (corr) {
-#pragma unroll
-    for (int c = 0; c < 6; ++c) cm[c] = corr_mean[c];
-  }
   for (int i = threadIdx.x; i < lines * N; i += blockDim.x) {
     const int x = i % N, ll = i / N;
     const long long lj = line0 + ll;
@@ -807,11 +791,7 @@ __global__ void __launch_bounds__(512) pass_x_a_kernel(typename C<R>::T* __restr
         e[2 * q + 1] += z.y;
       }
     }
-    if (corr) {
-#pragma unroll
-      for (int c = 0; c < 6; ++c) e[c] += (R)((double)corr[c * d.N + vv] - cm[c]);
-    }
-    if (have_delta || zero || corr) {
+    if (have_delta || zero) {
 #pragma unroll
       for (int c = 0; c < 6; ++c) eps[c * d.N + vv] = e[c];
     }

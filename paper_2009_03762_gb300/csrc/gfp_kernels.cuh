@@ -254,27 +254,32 @@ __device__ __forceinline__ double incr_norm2(const R d[6]) {
 
 // Block sum of one double per thread (thread 0 receives the result); all threads must call.
 __device__ __forceinline__ double block_sum(double v, double* red) {
-  for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+  const int lane = threadIdx.x & 31, wn = min(32, (int)(blockDim.x - (threadIdx.x & ~31u)));  // lanes of this warp
+  const unsigned mask = wn == 32 ? 0xffffffffu : (1u << wn) - 1u;
+  for (int off = 16; off > 0; off >>= 1) {
+    const double u = __shfl_down_sync(mask, v, off);
+    if (lane + off < wn) v += u;
+  }
+  if (lane == 0) red[threadIdx.x >> 5] = v;
   __syncthreads();
   double s = 0.0;
   if (threadIdx.x < 32) {
     const int nw = (blockDim.x + 31) >> 5;
-    s = threadIdx.x < nw ? red[threadIdx.x] : 0.0;
-    for (int off = 16; off > 0; off >>= 1) s += __shfl_down_sync(0xffffffffu, s, off);
+    s = lane < nw ? red[lane] : 0.0;
+    for (int off = 16; off > 0; off >>= 1) {
+      const double u = __shfl_down_sync(mask, s, off);
+      if (lane + off < wn) s += u;
+    }
   }
   return s;
 }
 
 // flags: PX_DELTA adds the inverse x-transform of the spectrum (the previous increment) to the state;
-// PX_ZERO starts from a zero state (not read, written as zeros).  corr (FP32, may be null) is an
-// additive correction with FP64 mean corr_mean removed: state += corr - corr_mean (mixed-precision
-// refinement of the FP64 strain).
+// PX_ZERO starts from a zero state (not read, written as zeros).
 template <typename R>
 __global__ void pass_x_kernel(typename C<R>::T* __restrict__ spec, R* __restrict__ eps, const R* __restrict__ lam,
                               const R* __restrict__ mu, const typename C<R>::T* __restrict__ tw, FftPlan plan, Dims d,
-                              int lines, int flags, const float* __restrict__ corr, const double* __restrict__ corr_mean,
-                              PolarParams pp, const SolveState* __restrict__ st) {
+                              int lines, int flags, PolarParams pp, const SolveState* __restrict__ st) {
   typedef typename C<R>::T T;
   if (st->done) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -319,11 +324,6 @@ __global__ void pass_x_kernel(typename C<R>::T* __restrict__ spec, R* __restrict
   } else {
     __syncthreads();
   }
-  double cm[6];
-  if (corr) {
-#pragma unroll
-    for (int c = 0; c < 6; ++c) cm[c] = corr_mean[c];
-  }
   const bool polar = (flags & PX_POLAR) != 0;
   const bool dres = sizeof(R) == 8 && (flags & PX_DRES) != 0;
   double dacc = 0.0;
@@ -361,11 +361,7 @@ __global__ void pass_x_kernel(typename C<R>::T* __restrict__ spec, R* __restrict
         for (int c = 0; c < 6; ++c) e[c] += dd[c];
       }
     }
-    if (corr) {
-#pragma unroll
-      for (int c = 0; c < 6; ++c) e[c] += (R)((double)corr[c * d.N + v] - cm[c]);
-    }
-    if (have_delta || zero || corr) {
+    if (have_delta || zero) {
 #pragma unroll
       for (int c = 0; c < 6; ++c) eps[c * d.N + v] = e[c];
     }
@@ -629,6 +625,13 @@ inline bool has_register_plan(int n) {
   return false;
 }
 
+// Twiddle table entries: FP32 passes read w_n^j as float2, FP64 passes (fixed-point transforms, gfp_fx.cuh) as
+// 2^62 w_n^j with each part split h 2^32 + l, l signed and above INT_MIN.
+struct __align__(16) fxw { int xh, xl, yh, yl; };
+template <typename R> struct TwT;
+template <> struct TwT<float> { typedef float2 type; };
+template <> struct TwT<double> { typedef fxw type; };
+
 struct LaunchCfg {
   int x_lines, x_threads;   // generic x-pass
   int y_cols, y_threads;
@@ -645,13 +648,14 @@ struct LaunchCfg {
 template <typename R>
 struct Passes {
   typedef typename C<R>::T T;
+  typedef typename TwT<R>::type W;
   static cudaError_t setup();   // opt-in shared memory limits
-  static void pass_x(cudaStream_t s, const LaunchCfg& lc, T* spec, R* eps, const R* lam, const R* mu, const T* tw,
-                     const FftPlan& plan, const Dims& d, int flags, const float* corr, const double* corr_mean,
+  static void pass_x(cudaStream_t s, const LaunchCfg& lc, T* spec, R* eps, const R* lam, const R* mu, const W* tw,
+                     const FftPlan& plan, const Dims& d, int flags,
                      const SolveState* st, const PolarParams* pp = nullptr);
-  static void pass_y(cudaStream_t s, const LaunchCfg& lc, bool inverse, T* spec, const T* tw, const FftPlan& plan,
+  static void pass_y(cudaStream_t s, const LaunchCfg& lc, bool inverse, T* spec, const W* tw, const FftPlan& plan,
                      const Dims& d, const SolveState* st, int comps = 6);
-  static void pass_z(cudaStream_t s, const LaunchCfg& lc, T* spec, const T* tw, const FftPlan& plan, const Dims& d,
+  static void pass_z(cudaStream_t s, const LaunchCfg& lc, T* spec, const W* tw, const FftPlan& plan, const Dims& d,
                      const GammaParams<R>& gp, double* partials, SolveState* st, int mode, float2* vsrc);
 };
 

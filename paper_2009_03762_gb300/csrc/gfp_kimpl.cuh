@@ -72,8 +72,8 @@ template <typename R, int N> inline int cx_lines_max() {
 
 template <typename R, int N>
 inline void launch_x_c(cudaStream_t s, int want_lines, int async, typename C<R>::T* spec, R* eps, const R* lam,
-                       const R* mu, const typename C<R>::T* tw, const Dims& d, int flags, const float* corr,
-                       const double* corr_mean, const PolarParams& pp, const SolveState* st) {
+                       const R* mu, const typename C<R>::T* tw, const Dims& d, int flags,
+                       const PolarParams& pp, const SolveState* st) {
   typedef typename C<R>::T T;
   if (async && !(flags & (PX_POLAR | PX_STRAIN | PX_OUTPUT | PX_DRES)) && !pp.estar) {
     int lines = want_lines > 0 ? want_lines : 2;
@@ -82,20 +82,19 @@ inline void launch_x_c(cudaStream_t s, int want_lines, int async, typename C<R>:
     const long long nlines = (long long)d.n2 * d.n3;
     const unsigned blocks = (unsigned)((nlines + lines - 1) / lines);
     pass_x_a_kernel<R, N><<<blocks, 3 * lines * CPlan<N>::T, xa_smem_bytes<R, N>(lines), s>>>(
-        spec, eps, lam, mu, tw, d, lines, flags, corr, corr_mean, st);
+        spec, eps, lam, mu, tw, d, lines, flags, st);
     return;
   }
   const int lines = want_lines > 0 ? std::min(want_lines, cx_lines_max<R, N>()) : cx_lines_max<R, N>();
   const long long nlines = (long long)d.n2 * d.n3;
   const unsigned blocks = (unsigned)((nlines + lines - 1) / lines);
   const size_t sm = cx_smem_bytes<R, N>(lines);
-  pass_x_c_kernel<R, N><<<blocks, 3 * lines * CPlan<N>::T, sm, s>>>(spec, eps, lam, mu, tw, d, lines, flags, corr,
-                                                                     corr_mean, pp, st);
+  pass_x_c_kernel<R, N><<<blocks, 3 * lines * CPlan<N>::T, sm, s>>>(spec, eps, lam, mu, tw, d, lines, flags, pp, st);
 }
 
 template <typename R>
-void Passes<R>::pass_x(cudaStream_t s, const LaunchCfg& lc, T* spec, R* eps, const R* lam, const R* mu, const T* tw,
-                       const FftPlan& plan, const Dims& d, int flags, const float* corr, const double* corr_mean,
+void Passes<R>::pass_x(cudaStream_t s, const LaunchCfg& lc, T* spec, R* eps, const R* lam, const R* mu, const W* tw,
+                       const FftPlan& plan, const Dims& d, int flags,
                        const SolveState* st, const PolarParams* ppp) {
   PolarParams pp;
   if (ppp) pp = *ppp;
@@ -107,7 +106,7 @@ void Passes<R>::pass_x(cudaStream_t s, const LaunchCfg& lc, T* spec, R* eps, con
   }
   switch (d.n1) {
 #define GFP_CASE(N) \
-    case N: launch_x_c<R, N>(s, lc.cx_lines, lc.x_async, spec, eps, lam, mu, tw, d, flags, corr, corr_mean, pp, st); return;
+    case N: launch_x_c<R, N>(s, lc.cx_lines, lc.x_async, spec, eps, lam, mu, tw, d, flags, pp, st); return;
     GFP_FOR_CSIZES(GFP_CASE)
 #undef GFP_CASE
     default: break;
@@ -115,12 +114,11 @@ void Passes<R>::pass_x(cudaStream_t s, const LaunchCfg& lc, T* spec, R* eps, con
   const long long nlines = (long long)d.n2 * d.n3;
   const unsigned blocks = (unsigned)((nlines + lc.x_lines - 1) / lc.x_lines);
   const size_t sm = sizeof(T) * (size_t)(d.n1 + 6 * lc.x_lines * d.n1);
-  pass_x_kernel<R><<<blocks, lc.x_threads, sm, s>>>(spec, eps, lam, mu, tw, plan, d, lc.x_lines, flags, corr,
-                                                     corr_mean, pp, st);
+  pass_x_kernel<R><<<blocks, lc.x_threads, sm, s>>>(spec, eps, lam, mu, tw, plan, d, lc.x_lines, flags, pp, st);
 }
 
 template <typename R>
-void Passes<R>::pass_y(cudaStream_t s, const LaunchCfg& lc, bool inverse, T* spec, const T* tw, const FftPlan& plan,
+void Passes<R>::pass_y(cudaStream_t s, const LaunchCfg& lc, bool inverse, T* spec, const W* tw, const FftPlan& plan,
                        const Dims& d, const SolveState* st, int comps) {
   dim3 grid((d.n1h + lc.y_cols - 1) / lc.y_cols, d.n3, comps);
   switch (d.n2) {
@@ -145,7 +143,7 @@ void Passes<R>::pass_y(cudaStream_t s, const LaunchCfg& lc, bool inverse, T* spe
 }
 
 template <typename R>
-void Passes<R>::pass_z(cudaStream_t s, const LaunchCfg& lc, T* spec, const T* tw, const FftPlan& plan, const Dims& d,
+void Passes<R>::pass_z(cudaStream_t s, const LaunchCfg& lc, T* spec, const W* tw, const FftPlan& plan, const Dims& d,
                        const GammaParams<R>& gp, double* partials, SolveState* st, int mode, float2* vsrc) {
   const int ntx = (d.n1h + lc.z_cols - 1) / lc.z_cols;
   dim3 grid(ntx, d.n2, 1);
