@@ -677,18 +677,25 @@ LaunchCfg make_cfg(const Dims& d, int eb) {
   while (L > 1 && (long long)(d.n1 + 6 * L * d.n1) * eb > budget) L /= 2;
   c.x_lines = L;
   c.x_threads = clampt(3 * L * d.n1 / 8);
-  int yc = eb == 16 ? 8 : 16;
+  // 128-byte rows, but half of that where a column takes 32 threads (FP64 at 256: 4 columns 0.503, 8 0.576 ms; FP32 at 512:
+  // 8 columns 1.20, 16 1.39 ms)
+  int yc = eb == 16 ? (d.n2 == 256 ? 4 : 8) : (d.n2 == 512 ? 8 : 16);
   while (yc > 1 && (long long)(d.n2 + 2 * yc * d.n2) * eb > budget) yc /= 2;
   c.y_cols = std::max(1, std::min(yc, d.n1h));
   c.y_threads = clampt(c.y_cols * d.n2 / 8);
-  int zc = d.n3 >= 512 ? 2 : 4;  // register-FFT z-pass: 6 zc (n3 / 16) threads <= 512
+  // register-FFT z-pass: 6 zc (n3 / 16) threads <= 512 (FP32 at 512: 4 columns 4.63, 2 columns 7.77 ms)
+  int zc = d.n3 >= 512 && (eb == 16 || d.n3 != 512) ? 2 : 4;
   while (zc > 1 && (long long)(d.n3 + 12 * zc * d.n3) * eb > budget) zc /= 2;
+  // the TMA-fed 8-column kernel at n3 = 256 where its tiles fill the chip twice (256^3: 0.295 against 0.411 ms; at n3 = 64, the
+  // other length it has, 12.3 us either way)
+  const bool tma8 = eb == 8 && d.n3 == 256 && d.n1h >= 8 && (long long)((d.n1h + 7) / 8) * d.n2 >= 304;
+  if (tma8) zc = 8;
   c.z_cols = std::max(1, std::min(zc, d.n1h));
   c.z_threads = clampt(6 * c.z_cols * d.n3 / 8);
   c.z_blocks = ((d.n1h + c.z_cols - 1) / c.z_cols) * d.n2;
   c.cx_lines = 0;
   c.ztmap = nullptr;
-  c.z_tma = 0;
+  c.z_tma = tma8 ? 1 : 0;
   c.x_async = 0;
   c.plan[0] = make_plan(d.n1);
   c.plan[1] = make_plan(d.n2);
@@ -764,14 +771,6 @@ bool encode_ztmap(CUtensorMap* m, const void* spec, const Dims& d, int cols, int
   return r == CUDA_SUCCESS;
 }
 
-// (Re)encode the z-tile tensor map of a launch configuration; without TMA the pass falls back to
-// the register-FFT kernel with ordinary loads.
-void refresh_ztmap(gfp_grid g, bool mixed) {
-  LaunchCfg& lc = mixed ? g->lc32 : g->lc64;
-  CUtensorMap* m = mixed ? &g->zmap32 : &g->zmap64;
-  lc.ztmap = encode_ztmap(m, g->spec, g->d, lc.z_cols, mixed ? 4 : 8) ? m : nullptr;
-}
-
 // Recompute the thread counts and partial-sum count after a tile change.
 void finalize_cfg(const Dims& d, LaunchCfg& c) {
   auto clampt = [](int t) { return std::min(512, std::max(64, round32(t))); };
@@ -779,6 +778,14 @@ void finalize_cfg(const Dims& d, LaunchCfg& c) {
   c.y_threads = clampt(c.y_cols * d.n2 / 8);
   c.z_threads = clampt(6 * c.z_cols * d.n3 / 8);
   c.z_blocks = ((d.n1h + c.z_cols - 1) / c.z_cols) * d.n2;
+}
+
+// (Re)encode the z-tile tensor map of a launch configuration; without TMA the pass falls back to
+// the register-FFT kernel with ordinary loads.
+void refresh_ztmap(gfp_grid g, bool mixed) {
+  LaunchCfg& lc = mixed ? g->lc32 : g->lc64;
+  CUtensorMap* m = mixed ? &g->zmap32 : &g->zmap64;
+  lc.ztmap = encode_ztmap(m, g->spec, g->d, lc.z_cols, mixed ? 4 : 8) ? m : nullptr;
 }
 
 // Per-axis tables with exact zeros (kappa from the storage index; Nyquist is kappa = -n/2)

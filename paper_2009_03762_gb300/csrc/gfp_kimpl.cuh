@@ -85,7 +85,9 @@ inline void launch_x_c(cudaStream_t s, int want_lines, int async, typename C<R>:
         spec, eps, lam, mu, tw, d, lines, flags, st);
     return;
   }
-  const int lines = want_lines > 0 ? std::min(want_lines, cx_lines_max<R, N>()) : cx_lines_max<R, N>();
+  // default: 96 threads a CTA, ten of them per SM at 64 registers (256^3, lines per CTA: 1 0.407, 2 0.347, 4 0.357, 10
+  // 0.434 ms; 192^3: 4 0.221, 16 0.315 ms; 128^3: 4 0.048, 16 0.056 ms)
+  const int lines = std::min(want_lines > 0 ? want_lines : std::max(1, 32 / CPlan<N>::T), cx_lines_max<R, N>());
   const long long nlines = (long long)d.n2 * d.n3;
   const unsigned blocks = (unsigned)((nlines + lines - 1) / lines);
   const size_t sm = cx_smem_bytes<R, N>(lines);
