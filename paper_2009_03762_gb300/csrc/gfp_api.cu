@@ -688,7 +688,7 @@ LaunchCfg make_cfg(const Dims& d, int eb) {
   while (zc > 1 && (long long)(d.n3 + 12 * zc * d.n3) * eb > budget) zc /= 2;
   // the TMA-fed 8-column kernel at n3 = 256 where its tiles fill the chip twice (256^3: 0.295 against 0.411 ms; at n3 = 64, the
   // other length it has, 12.3 us either way)
-  const bool tma8 = eb == 8 && d.n3 == 256 && d.n1h >= 8 && (long long)((d.n1h + 7) / 8) * d.n2 >= 304;
+  const bool tma8 = eb == 8 && (d.n3 == 256 || d.n3 == 512) && d.n1h >= 8 && (long long)((d.n1h + 7) / 8) * d.n2 >= 304;
   if (tma8) zc = 8;
   c.z_cols = std::max(1, std::min(zc, d.n1h));
   c.z_threads = clampt(6 * c.z_cols * d.n3 / 8);
@@ -786,6 +786,11 @@ void refresh_ztmap(gfp_grid g, bool mixed) {
   LaunchCfg& lc = mixed ? g->lc32 : g->lc64;
   CUtensorMap* m = mixed ? &g->zmap32 : &g->zmap64;
   lc.ztmap = encode_ztmap(m, g->spec, g->d, lc.z_cols, mixed ? 4 : 8) ? m : nullptr;
+  if (!lc.ztmap && mixed && g->d.n3 == 512 && lc.z_cols == 8) {  // only the TMA-fed kernel has this width
+    lc.z_cols = 4;
+    lc.z_tma = 0;
+    finalize_cfg(g->d, lc);
+  }
 }
 
 // Per-axis tables with exact zeros (kappa from the storage index; Nyquist is kappa = -n/2)
@@ -2192,9 +2197,10 @@ int gfp_set_tiles(gfp_grid g, int prec, const int tiles[3]) {
   const int zc = tiles[2] < 0 ? -tiles[2] : tiles[2];
   const bool zc_ok = mixed ? cz_cols_ok<float>(d.n3, zc) : cz_cols_ok<double>(d.n3, zc);
   const int xl = tiles[0] < 0 ? -tiles[0] : tiles[0];
+  const bool tall = mixed && d.n3 == 512 && tiles[2] == -8;  // the TMA-fed kernel of 512 rows
   if (xl > 16 || tiles[1] < 1 || tiles[1] > ycmax || tiles[1] > d.n1h || zc < 1 ||
-      !zc_ok || zc > d.n1h || (long long)(d.n2 + 2 * tiles[1] * d.n2) * eb > budget ||
-      (long long)(d.n3 + 12 * zc * d.n3) * eb > budget)
+      (!zc_ok && !tall) || zc > d.n1h || (long long)(d.n2 + 2 * tiles[1] * d.n2) * eb > budget ||
+      (!tall && (long long)(d.n3 + 12 * zc * d.n3) * eb > budget))
     return GFP_ERR_ARG;
   LaunchCfg& lc = mixed ? g->lc32 : g->lc64;
   lc.cx_lines = xl;

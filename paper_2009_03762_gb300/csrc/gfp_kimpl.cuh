@@ -32,6 +32,8 @@ cudaError_t Passes<R>::setup() {
     if (e == cudaSuccess) e = cudaFuncSetAttribute(pass_z_s_kernel<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
   GFP_FOR_CSIZES(GFP_SET_TMA)
 #undef GFP_SET_TMA
+  if (sizeof(R) == 4 && e == cudaSuccess)
+    e = cudaFuncSetAttribute(pass_z_l_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ZL::smem);
   return e;
 }
 
@@ -159,6 +161,13 @@ void Passes<R>::pass_z(cudaStream_t s, const LaunchCfg& lc, T* spec, const W* tw
           pass_z_s_kernel<N><<<grid, 24 * CPlan<N>::T, zs_smem_bytes<N>(), s>>>(                              \
               *reinterpret_cast<const CUtensorMap*>(lc.ztmap), reinterpret_cast<const float2*>(tw), d,        \
               *reinterpret_cast<const GammaParams<float>*>(&gp), partials, st, vsrc);                         \
+          return;                                                                                             \
+        }                                                                                                     \
+      }                                                                                                       \
+      if constexpr (sizeof(R) == 4 && N == ZL::LEN) {                                                           \
+        if (mode == PZ_INNER && lc.z_tma && lc.ztmap && lc.z_cols == ZL::COLS && !gp.nyq_avg) {               \
+          pass_z_l_kernel<<<grid, ZL::NT, ZL::smem, s>>>(*reinterpret_cast<const CUtensorMap*>(lc.ztmap),     \
+              reinterpret_cast<const float2*>(tw), d, *reinterpret_cast<const GammaParams<float>*>(&gp), partials, st, vsrc); \
           return;                                                                                             \
         }                                                                                                     \
       }                                                                                                       \

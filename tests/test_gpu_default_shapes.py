@@ -1,4 +1,4 @@
-"""The launch shapes that grids take by default, in mixed precision: against the FP64 GPU solve (the bar of the mixed solve, 1e-6 relative)."""
+"""The launch shapes that grids take by default, and the z-pass of 512 rows, in mixed precision: against the FP64 GPU solve (the bar of the mixed solve, 1e-6 relative)."""
 import numpy as np
 import pytest
 
@@ -34,6 +34,11 @@ def _check(gfp, shape, tiles=None):
     assert _rel(eps, g.strain()) <= 1e-6
     assert _rel(r.sigma_mean, r64.sigma_mean) <= 1e-6
     g.close()
+
+
+@pytest.mark.parametrize("n1", [16, 18, 32, 54])  # 9, 10, 17 and 28 columns of the half spectrum
+def test_tall_tiles(gfp, n1):
+    _check(gfp, (n1, 6, 512), [2, 4, -8])
 
 
 @pytest.mark.parametrize("shape", [(64, 64, 256), (64, 64, 512), (32, 512, 8), (512, 8, 8), (192, 12, 8), (8, 8, 512)])
