@@ -672,20 +672,29 @@ LaunchCfg make_cfg(const Dims& d, int eb) {
   const long long budget = 200 * 1024;
   auto clampt = [](int t) { return std::min(512, std::max(64, round32(t))); };
   LaunchCfg c;
-  int L = std::max(1, std::min(16, 2048 / d.n1));
-  L = (int)std::min<long long>(L, (long long)d.n2 * d.n3);
+  // lengths without a register plan: about 400 elements of x a CTA, so that three or more share an SM (162^3 FP32 x-pass: 2 lines
+  // 227, 12 lines 328 us; FP64 81^3: 4 lines 94, 16 lines 118 us), fewer while the CTAs would not fill the chip twice
+  int L = std::max(1, std::min(4, 400 / d.n1));
+  while (L > 1 && (long long)d.n2 * d.n3 / L < 304) L /= 2;
   while (L > 1 && (long long)(d.n1 + 6 * L * d.n1) * eb > budget) L /= 2;
   c.x_lines = L;
   c.x_threads = clampt(3 * L * d.n1 / 8);
   // 128-byte rows, but half of that where a column takes 32 threads (FP64 at 256: 4 columns 0.503, 8 0.576 ms; FP32 at 512:
   // 8 columns 1.20, 16 1.39 ms)
   int yc = eb == 16 ? (d.n2 == 256 ? 4 : 8) : (d.n2 == 512 ? 8 : 16);
+  // lengths without a register plan: smaller tiles, more CTAs (FP32 162^3: 4 columns 131, 16 153 us; 108^3: 8 columns 33, 16 41;
+  // FP64 162^3: 4 columns 449, 8 525 us)
+  if (!has_register_plan(d.n2)) yc = d.n2 > 128 ? 4 : 8;
   while (yc > 1 && (long long)(d.n2 + 2 * yc * d.n2) * eb > budget) yc /= 2;
   c.y_cols = std::max(1, std::min(yc, d.n1h));
   c.y_threads = clampt(c.y_cols * d.n2 / 8);
   // register-FFT z-pass: 6 zc (n3 / 16) threads <= 512 (FP32 at 512: 4 columns 4.63, 2 columns 7.77 ms)
   int zc = d.n3 >= 512 && (eb == 16 || d.n3 != 512) ? 2 : 4;
   while (zc > 1 && (long long)(d.n3 + 12 * zc * d.n3) * eb > budget) zc /= 2;
+  // lengths without a register plan: 2 columns (FP32 162^3: 239 us, 4 columns 344; FP64 162^3 834 against 903, 54^3 37 against 61
+  // us), one where those CTAs would not fill the chip twice or a column is long (FP64 243^3: 2945 against 3222 us)
+  if (!has_register_plan(d.n3))
+    zc = (long long)((d.n1h + 1) / 2) * d.n2 < 304 || (eb == 16 && d.n3 > 200) || zc < 2 ? 1 : 2;
   // the TMA-fed 8-column kernel at n3 = 256 where its tiles fill the chip twice (256^3: 0.295 against 0.411 ms; at n3 = 64, the
   // other length it has, 12.3 us either way)
   const bool tma8 = eb == 8 && (d.n3 == 256 || d.n3 == 512) && d.n1h >= 8 && (long long)((d.n1h + 7) / 8) * d.n2 >= 304;
@@ -1142,12 +1151,12 @@ void outer_source32(cudaStream_t s, const LaunchCfg& lc32, const Dims& d, int op
   const long long nlines = (long long)d.n2 * d.n3;
   const int L = 4;
   const size_t smx = sizeof(float2) * 2 * (3 * L / 2) * (size_t)d.n1;
-  rx_kernel<<<(unsigned)((nlines + L - 1) / L), 256, smx, s>>>(rbuf, vsrc, tw32[0], lc32.plan[0], d, L, st);
+  rx_kernel<<<(unsigned)((nlines + L - 1) / L), 256, smx, s>>>(rbuf, vsrc, tw32[0], merge_stages(lc32.plan[0]), d, L, st);
   Passes<float>::pass_y(s, lc32, false, vsrc, tw32[1], lc32.plan[1], d, st, 3);
   const int zc = rz_cols(d.n3);
   const size_t smz = sizeof(float2) * 2 * (size_t)zc * (d.n3 + 1);
   const bool phase = res_stencil(op) == RS_AFD;
-  rz_kernel<<<dim3((d.n1h + zc - 1) / zc, d.n2, 3), 256, smz, s>>>(vsrc, tw32[2], lc32.plan[2], d, zc,
+  rz_kernel<<<dim3((d.n1h + zc - 1) / zc, d.n2, 3), 256, smz, s>>>(vsrc, tw32[2], merge_stages(lc32.plan[2]), d, zc,
                                                                    phase ? ph[0] : nullptr, phase ? ph[1] : nullptr,
                                                                    phase ? ph[2] : nullptr, st);
   launches += 3;

@@ -2,7 +2,7 @@
 //
 // The 3D transforms of the solver (eq. DisFouMat3D: a product of 1D transforms along x1, x2, x3)
 // are done one axis per pass.  Each pass stages a tile of complete lines in shared memory and runs
-// the 1D transform on all of them: radix stages (2, 3, 4, 8, 16) in Stockham autosort order, each
+// the 1D transform on all of them: radix stages (2, 3, 4, 8, 16 and products up to 18) in Stockham autosort order, each
 // thread holding its butterflies in registers between one shared-memory read and one write.
 //
 // Sign and scale: forward uses e^{-2 pi i jk/n}, inverse e^{+2 pi i jk/n}, both unnormalised; the
@@ -146,6 +146,45 @@ template <bool INV, typename T> struct Dft<16, INV, T> {
   }
 };
 
+// cos(2 pi j / 36), from the first quadrant (compile-time j)
+__host__ __device__ constexpr double cos36(int j) {
+  constexpr double c[10] = {1.0, 0.98480775301220805936, 0.93969262078590838405, 0.86602540378443864676,
+                            0.76604444311897803520, 0.64278760968653932632, 0.5, 0.34202014332566873304,
+                            0.17364817766693034885, 0.0};
+  j = j % 36 < 0 ? j % 36 + 36 : j % 36;
+  return j <= 9 ? c[j] : (j <= 18 ? -c[18 - j] : (j <= 27 ? -c[j - 18] : c[36 - j]));
+}
+// N = A B: columns x[p + B q], twiddles w_N^{p k1}, rows: X[k1 + A k2] = sum_p w_B^{p k2} w_N^{p k1} DFT_A(column p)[k1]
+template <int A, int B, bool INV, typename T> __device__ __forceinline__ void dft_composite(T* v) {
+  typedef decltype(T().x) R;
+  T y[B][A];
+#pragma unroll
+  for (int p = 0; p < B; ++p) {
+#pragma unroll
+    for (int q = 0; q < A; ++q) y[p][q] = v[p + B * q];
+    Dft<A, INV, T>::run(y[p]);
+  }
+#pragma unroll
+  for (int k1 = 0; k1 < A; ++k1) {
+    T z[B];
+#pragma unroll
+    for (int p = 0; p < B; ++p) {
+      const int j = 36 / (A * B) * p * k1;
+      T w;
+      w.x = (R)cos36(j);
+      w.y = (R)(INV ? cos36(9 - j) : -cos36(9 - j));
+      z[p] = p * k1 == 0 ? y[p][k1] : cmul(y[p][k1], w);
+    }
+    Dft<B, INV, T>::run(z);
+#pragma unroll
+    for (int k2 = 0; k2 < B; ++k2) v[k1 + A * k2] = z[k2];
+  }
+}
+template <bool INV, typename T> struct Dft<6, INV, T> { __device__ __forceinline__ static void run(T* v) { dft_composite<3, 2, INV>(v); } };
+template <bool INV, typename T> struct Dft<9, INV, T> { __device__ __forceinline__ static void run(T* v) { dft_composite<3, 3, INV>(v); } };
+template <bool INV, typename T> struct Dft<12, INV, T> { __device__ __forceinline__ static void run(T* v) { dft_composite<4, 3, INV>(v); } };
+template <bool INV, typename T> struct Dft<18, INV, T> { __device__ __forceinline__ static void run(T* v) { dft_composite<9, 2, INV>(v); } };
+
 // ---------------------------------------------------------------- FFT plan
 struct FftPlan {
   int n;
@@ -161,6 +200,41 @@ struct LineLayout {
   bool line_fast;
 };
 
+// q / d for q d < 2^32 by a multiplication (the stages divide once or twice per butterfly).
+struct FastDiv {
+  unsigned d, m;
+  __device__ __forceinline__ explicit FastDiv(int n) : d((unsigned)n), m(0xffffffffu / (unsigned)n + 1u) {}
+  __device__ __forceinline__ int div(int q) const { return d == 1u ? q : (int)__umulhi((unsigned)q, m); }
+};
+
+// The stages a schedule runs as: neighbouring stages merged while their product is one of the radices below, in the least
+// number of stages (each stage crosses shared memory twice; 162 = 2 3 3 3 3 runs as 18 9).
+inline FftPlan merge_stages(const FftPlan& p) {
+  auto ok = [](int r) { return r == 2 || r == 3 || r == 4 || r == 6 || r == 8 || r == 9 || r == 12 || r == 16 || r == 18; };
+  int best[13], from[13];
+  best[0] = 0;
+  for (int e = 1; e <= p.nst; ++e) {
+    best[e] = 1 << 20;
+    from[e] = e - 1;
+    int prod = 1;
+    for (int b = e - 1; b >= 0; --b) {
+      prod *= p.radix[b];
+      if (prod > 18) break;
+      if (ok(prod) && best[b] + 1 < best[e]) { best[e] = best[b] + 1; from[e] = b; }
+    }
+  }
+  FftPlan m;
+  m.n = p.n;
+  m.nst = best[p.nst];
+  for (int e = p.nst, s = m.nst - 1; e > 0; e = from[e], --s) {
+    int prod = 1;
+    for (int b = from[e]; b < e; ++b) prod *= p.radix[b];
+    m.radix[s] = prod;
+  }
+  for (int s = m.nst; s < 12; ++s) m.radix[s] = 0;
+  return m;
+}
+
 // One Stockham stage with radix RADIX, out of place (src -> dst): butterfly j of a line reads
 // elements j + r n/RADIX, multiplies element r by w_n^{r k n/(Ns RADIX)} (k = j mod Ns), transforms,
 // and writes element r to (j / Ns) Ns RADIX + k + r Ns.
@@ -170,15 +244,15 @@ __device__ __forceinline__ void fft_stage(const T* __restrict__ src, T* __restri
   const int nb = n / RADIX;
   const int total = L.lines * nb;
   const int tstride = n / (Ns * RADIX);
+  const FastDiv by_line(L.line_fast ? L.lines : nb), by_ns(Ns);
   for (int t = threadIdx.x; t < total; t += blockDim.x) {
-    int l, j;
-    if (L.line_fast) { l = t % L.lines; j = t / L.lines; }
-    else { j = t % nb; l = t / nb; }
+    const int hi = by_line.div(t), lo = t - hi * (int)by_line.d;
+    const int l = L.line_fast ? lo : hi, j = L.line_fast ? hi : lo;
     const T* sb = src + l * L.ls;
     T v[RADIX];
 #pragma unroll
     for (int r = 0; r < RADIX; ++r) v[r] = sb[(j + r * nb) * L.es];
-    const int k = j % Ns;
+    const int jn = by_ns.div(j), k = j - jn * Ns;
     if (k > 0) {
 #pragma unroll
       for (int r = 1; r < RADIX; ++r) {
@@ -189,7 +263,7 @@ __device__ __forceinline__ void fft_stage(const T* __restrict__ src, T* __restri
     }
     Dft<RADIX, INV, T>::run(v);
     T* db = dst + l * L.ls;
-    const int o = (j / Ns) * Ns * RADIX + k;
+    const int o = jn * Ns * RADIX + k;
 #pragma unroll
     for (int r = 0; r < RADIX; ++r) db[(o + r * Ns) * L.es] = v[r];
   }
@@ -211,7 +285,11 @@ __device__ __forceinline__ T* fft_lines(T* a, T* b, const T* tw, const FftPlan& 
       case 2: fft_stage<2, INV>(src, dst, tw, P.n, Ns, L); break;
       case 3: fft_stage<3, INV>(src, dst, tw, P.n, Ns, L); break;
       case 4: fft_stage<4, INV>(src, dst, tw, P.n, Ns, L); break;
+      case 6: fft_stage<6, INV>(src, dst, tw, P.n, Ns, L); break;
       case 8: fft_stage<8, INV>(src, dst, tw, P.n, Ns, L); break;
+      case 9: fft_stage<9, INV>(src, dst, tw, P.n, Ns, L); break;
+      case 12: fft_stage<12, INV>(src, dst, tw, P.n, Ns, L); break;
+      case 18: fft_stage<18, INV>(src, dst, tw, P.n, Ns, L); break;
       default: fft_stage<16, INV>(src, dst, tw, P.n, Ns, L); break;
     }
     Ns *= R;

@@ -66,7 +66,7 @@ __device__ __forceinline__ fx2 fx_twiddle(fx2 a, fxw w) {
   return r;
 }
 
-// Small transforms; those of radix 6 to 16 scale by 1/4 between their two layers.
+// Small transforms; those of radix 6 to 16 scale by 1/4 between their two layers, radix 18 by 1/8 in all.
 template <int RADIX, bool INV> struct FxDft {
   __device__ __forceinline__ static void run(fx2* v) { Dft<RADIX, INV, fx2>::run(v); }
 };
@@ -151,57 +151,50 @@ template <bool INV> struct FxDft<16, INV> {
   }
 };
 
-// w12^j = e^{-+ 2 pi i j / 12}, j = 1, 2, 4 (Q62)
-__device__ __forceinline__ fxw fx_w12(int j, bool inv) {
-  constexpr int ch = 929887697, cl = -1332128537, half = 1 << 29;  // sqrt(3)/2 and 1/2
+// e^{-+ 2 pi i j / 36} (Q62, split; compile-time j)
+__device__ __forceinline__ fxw fx_w36(int j, bool inv) {
+  constexpr long long c[10] = {4611686018427387904LL, 4541624145405292212LL, 4333567320897763126LL, 3993837246235628775LL,
+                               3532756447825785444LL, 2964334632409774423LL, 2305843009213693952LL, 1577289512995517789LL,
+                               800810873071977681LL,  0LL};
+  auto cs = [&](int i) -> long long {
+    i = (i % 36 + 36) % 36;
+    return i <= 9 ? c[i] : (i <= 18 ? -c[18 - i] : (i <= 27 ? -c[i - 18] : c[36 - i]));
+  };
+  const long long x = cs(j), y = inv ? cs(9 - j) : -cs(9 - j);
   fxw w;
-  w.xh = j == 1 ? ch : (j == 2 ? half : -half); w.xl = j == 1 ? cl : 0;
-  w.yh = j == 1 ? half : ch;                    w.yl = j == 1 ? 0 : cl;
-  if (!inv) { w.yh = -w.yh; w.yl = -w.yl; }
+  w.xl = (int)x; w.xh = fx_high(x);
+  w.yl = (int)y; w.yh = fx_high(y);
   return w;
 }
-template <bool INV> struct FxDft<6, INV> {  // 6 = 3 x 2
-  __device__ __forceinline__ static void run(fx2* v) {
-    fx2 a[3] = {v[0], v[2], v[4]}, b[3] = {v[1], v[3], v[5]};
-    FxDft<3, INV>::run(a);
-    FxDft<3, INV>::run(b);
-    b[0] = fx_shr<2>(b[0]);
-    b[1] = fx_cmul<false>(b[1], fx_w12(2, INV));
-    b[2] = fx_cmul<false>(b[2], fx_w12(4, INV));
+// As dft_composite, with the elements scaled down by S bits between the layers.
+template <int A, int B, bool INV, int S> __device__ __forceinline__ void fx_composite(fx2* v) {
+  fx2 y[B][A];
 #pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      const fx2 s = fx_shr<2>(a[k]);
-      v[k] = cadd(s, b[k]);
-      v[k + 3] = csub(s, b[k]);
-    }
+  for (int p = 0; p < B; ++p) {
+#pragma unroll
+    for (int q = 0; q < A; ++q) y[p][q] = v[p + B * q];
+    FxDft<A, INV>::run(y[p]);
   }
-};
-template <bool INV> struct FxDft<12, INV> {  // 12 = 4 x 3: columns p, twiddles w12^{p k1}, rows k1
-  __device__ __forceinline__ static void run(fx2* v) {
-    fx2 y[3][4];
 #pragma unroll
-    for (int p = 0; p < 3; ++p) {
+  for (int k1 = 0; k1 < A; ++k1) {
+    fx2 z[B];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) y[p][q] = v[p + 3 * q];
-      Dft<4, INV, fx2>::run(y[p]);
+    for (int p = 0; p < B; ++p) {
+      const int j = 36 / (A * B) * p * k1;
+      if (j == 0) z[p] = fx_shr<S>(y[p][k1]);
+      else if (j == 9) z[p] = fx_shr<S>(mul_mi<INV>(y[p][k1]));
+      else z[p] = fx_twiddle<false, S>(y[p][k1], fx_w36(j, INV));
     }
+    FxDft<B, INV>::run(z);
 #pragma unroll
-    for (int k1 = 0; k1 < 4; ++k1) {
-      fx2 z[3];
-#pragma unroll
-      for (int p = 0; p < 3; ++p) {
-        const int j = p * k1;
-        if (j == 0) z[p] = fx_shr<2>(y[p][k1]);
-        else if (j == 3) z[p] = fx_shr<2>(mul_mi<INV>(y[p][k1]));
-        else if (j == 6) { z[p] = fx_shr<2>(y[p][k1]); z[p].x = fx_sub(0, z[p].x); z[p].y = fx_sub(0, z[p].y); }
-        else z[p] = fx_cmul<false>(y[p][k1], fx_w12(j, INV));
-      }
-      FxDft<3, INV>::run(z);
-#pragma unroll
-      for (int k2 = 0; k2 < 3; ++k2) v[k1 + 4 * k2] = z[k2];
-    }
+    for (int k2 = 0; k2 < B; ++k2) v[k1 + A * k2] = z[k2];
   }
-};
+}
+// (moduli from 2^60.5: radix 3 to 2^62.1, / 4, x 3 or x 2; radix 9 leaves 2^61.7, / 2, x 2)
+template <bool INV> struct FxDft<6, INV> { __device__ __forceinline__ static void run(fx2* v) { fx_composite<3, 2, INV, 2>(v); } };
+template <bool INV> struct FxDft<9, INV> { __device__ __forceinline__ static void run(fx2* v) { fx_composite<3, 3, INV, 2>(v); } };
+template <bool INV> struct FxDft<12, INV> { __device__ __forceinline__ static void run(fx2* v) { fx_composite<4, 3, INV, 2>(v); } };
+template <bool INV> struct FxDft<18, INV> { __device__ __forceinline__ static void run(fx2* v) { fx_composite<9, 2, INV, 1>(v); } };
 
 // Register plans of the fixed-point transforms.  An element takes four registers, so a thread holds 8 of them (about 80
 // registers and 24 warps per SM; 16 elements per thread took 136-176 registers and left the integer pipes waiting), and
@@ -233,7 +226,7 @@ template <int N, int S> __device__ __forceinline__ int fout_idx(int t, int b, in
 // Bits by which the elements are scaled down before the stage that follows one of radix R, and inside
 // a stage of radix R.
 __host__ __device__ constexpr int fx_post(int R) { return R == 8 || R == 6 || R == 2 ? 1 : 2; }
-__host__ __device__ constexpr int fx_inner(int R) { return R >= 6 ? 2 : 0; }
+__host__ __device__ constexpr int fx_inner(int R) { return R == 18 ? 3 : (R >= 6 ? 2 : 0); }
 template <int N> __host__ __device__ constexpr int fx_shift() {
   typedef FxPlan<N> P;
   int s = 0;
@@ -1186,15 +1179,15 @@ template <int RADIX, bool INV>
 __device__ __forceinline__ void fx_stage_lines(const fx2* __restrict__ src, fx2* __restrict__ dst, const fxw* __restrict__ tw,
                                                int n, int Ns, int post, LineLayout L) {
   const int nb = n / RADIX, total = L.lines * nb, tstride = n / (Ns * RADIX);
+  const FastDiv by_line(L.line_fast ? L.lines : nb), by_ns(Ns);
   for (int q = threadIdx.x; q < total; q += blockDim.x) {
-    int l, j;
-    if (L.line_fast) { l = q % L.lines; j = q / L.lines; }
-    else { j = q % nb; l = q / nb; }
+    const int hi = by_line.div(q), lo = q - hi * (int)by_line.d;
+    const int l = L.line_fast ? lo : hi, j = L.line_fast ? hi : lo;
     const fx2* sb = src + l * L.ls;
     fx2 v[RADIX];
 #pragma unroll
     for (int r = 0; r < RADIX; ++r) v[r] = sb[(j + r * nb) * L.es];
-    const int k = j % Ns;
+    const int jn = by_ns.div(j), k = j - jn * Ns;
     if (post) {
       v[0] = post == 1 ? fx_shr<1>(v[0]) : fx_shr<2>(v[0]);
 #pragma unroll
@@ -1205,7 +1198,7 @@ __device__ __forceinline__ void fx_stage_lines(const fx2* __restrict__ src, fx2*
     }
     FxDft<RADIX, INV>::run(v);
     fx2* db = dst + l * L.ls;
-    const int o = (j / Ns) * Ns * RADIX + k;
+    const int o = jn * Ns * RADIX + k;
 #pragma unroll
     for (int r = 0; r < RADIX; ++r) db[(o + r * Ns) * L.es] = v[r];
   }
@@ -1223,7 +1216,11 @@ __device__ __forceinline__ fx2* fx_lines(fx2* a, fx2* b, const fxw* tw, const Ff
       case 2: fx_stage_lines<2, INV>(src, dst, tw, P.n, Ns, post, L); break;
       case 3: fx_stage_lines<3, INV>(src, dst, tw, P.n, Ns, post, L); break;
       case 4: fx_stage_lines<4, INV>(src, dst, tw, P.n, Ns, post, L); break;
+      case 6: fx_stage_lines<6, INV>(src, dst, tw, P.n, Ns, post, L); break;
       case 8: fx_stage_lines<8, INV>(src, dst, tw, P.n, Ns, post, L); break;
+      case 9: fx_stage_lines<9, INV>(src, dst, tw, P.n, Ns, post, L); break;
+      case 12: fx_stage_lines<12, INV>(src, dst, tw, P.n, Ns, post, L); break;
+      case 18: fx_stage_lines<18, INV>(src, dst, tw, P.n, Ns, post, L); break;
       default: fx_stage_lines<16, INV>(src, dst, tw, P.n, Ns, post, L); break;
     }
     Ns *= R;
@@ -1238,8 +1235,9 @@ __device__ __forceinline__ fx2* fx_lines(fx2* a, fx2* b, const fxw* tw, const Ff
 template <int BITS>
 __device__ __forceinline__ void fx_tile_in(double2* buf, int* emax, int n, LineLayout L) {
   const int per = max(1, (int)blockDim.x / L.lines);  // threads per line, each on every per-th element
+  const FastDiv by_per(L.line_fast ? L.lines : per), by_n(L.line_fast ? L.lines : n);
   for (int q = threadIdx.x; q < per * L.lines; q += blockDim.x) {
-    const int l = L.line_fast ? q % L.lines : q / per, c = L.line_fast ? q / L.lines : q % per;
+    const int hi = by_per.div(q), lo = q - hi * (int)by_per.d, l = L.line_fast ? lo : hi, c = L.line_fast ? hi : lo;
     int m = 0;
     for (int e = c; e < n; e += per) {
       const double2 w = buf[l * L.ls + e * L.es];
@@ -1249,7 +1247,7 @@ __device__ __forceinline__ void fx_tile_in(double2* buf, int* emax, int n, LineL
   }
   __syncthreads();
   for (int q = threadIdx.x; q < n * L.lines; q += blockDim.x) {
-    const int l = L.line_fast ? q % L.lines : q / n, e = L.line_fast ? q / L.lines : q % n;
+    const int hi = by_n.div(q), lo = q - hi * (int)by_n.d, l = L.line_fast ? lo : hi, e = L.line_fast ? hi : lo;
     const FxLine F = fx_line(emax[l]);
     double2* at = buf + l * L.ls + e * L.es;
     double2 w = *at;
@@ -1274,12 +1272,13 @@ __global__ void __launch_bounds__(512) pass_y_fxg_kernel(double2* __restrict__ s
   double2* buf = reinterpret_cast<double2*>(twl + d.n2);  // [n2][cols], two ping-pong copies
   __shared__ int emax[64];
   const int k10 = blockIdx.x * cols;
+  const FastDiv by_cols(cols);
   for (int i = threadIdx.x; i < d.n2; i += blockDim.x) twl[i] = tw[i];
   for (int i = threadIdx.x; i < cols; i += blockDim.x) emax[i] = 0;
   double2* g = spec + blockIdx.z * d.S + d.row(blockIdx.y, 0) * d.P + k10;
   const long long ys = d.ystride();
   for (int i = threadIdx.x; i < d.n2 * cols; i += blockDim.x) {
-    const int cc = i % cols, y = i / cols;
+    const int y = by_cols.div(i), cc = i - y * cols;
     buf[i] = k10 + cc < d.n1h ? g[y * ys + cc] : make_double2(0.0, 0.0);
   }
   __syncthreads();
@@ -1288,7 +1287,7 @@ __global__ void __launch_bounds__(512) pass_y_fxg_kernel(double2* __restrict__ s
   const fx2* r = fx_lines<INV>(reinterpret_cast<fx2*>(buf), reinterpret_cast<fx2*>(buf + d.n2 * cols), twl, plan, L);
   const int sh = fx_shift(plan);
   for (int i = threadIdx.x; i < d.n2 * cols; i += blockDim.x) {
-    const int cc = i % cols, y = i / cols;
+    const int y = by_cols.div(i), cc = i - y * cols;
     if (k10 + cc >= d.n1h) continue;
     const FxLine F = fx_line(emax[cc]);
     g[y * ys + cc] = fx_out(r[i], fx_bias<60>(F, sh, 0), F);
@@ -1313,12 +1312,13 @@ __global__ void __launch_bounds__(512) pass_x_fxg_kernel(double2* __restrict__ s
   const bool outmode = (flags & PX_OUTPUT) != 0, strainmode = (flags & PX_STRAIN) != 0;
   const bool polar = (flags & PX_POLAR) != 0, dres = (flags & PX_DRES) != 0;
   const LineLayout L{tot, 1, n1, false};
+  const FastDiv by_n(n1), by_h(n1h), by_lines(lines);
   for (int i = threadIdx.x; i < n1; i += blockDim.x) twl[i] = tw[i];
   for (int i = threadIdx.x; i < 2 * tot; i += blockDim.x) emax[i / tot][i % tot] = 0;
   fx2* inc = reinterpret_cast<fx2*>(bufa);
   if (have_delta) {
     for (int i = threadIdx.x; i < tot * n1h; i += blockDim.x) {
-      const int k = i % n1h, pl = i / n1h, l = pl % lines, p = pl / lines;
+      const int pl = by_h.div(i), k = i - pl * n1h, p = by_lines.div(pl), l = pl - p * lines;
       const long long li = line0 + l;
       double2 z0 = make_double2(0.0, 0.0), z1 = z0;
       if (li < nlines) {
@@ -1341,7 +1341,7 @@ __global__ void __launch_bounds__(512) pass_x_fxg_kernel(double2* __restrict__ s
   double2* sig = reinterpret_cast<double2*>(inc);
   double dacc = 0.0;
   for (int i = threadIdx.x; i < lines * n1; i += blockDim.x) {
-    const int x = i % n1, l = i / n1;
+    const int l = by_n.div(i), x = i - l * n1;
     const long long li = line0 + l;
     if (li >= nlines) {
       for (int p = 0; p < 3; ++p) sig[(p * lines + l) * n1 + x] = make_double2(0.0, 0.0);
@@ -1402,12 +1402,12 @@ __global__ void __launch_bounds__(512) pass_x_fxg_kernel(double2* __restrict__ s
   double2* other = sig == bufa ? bufb : bufa;
   const fx2* Z = fx_lines<false>(reinterpret_cast<fx2*>(sig), reinterpret_cast<fx2*>(other), twl, plan, L);
   for (int i = threadIdx.x; i < tot * n1h; i += blockDim.x) {
-    const int k = i % n1h, pl = i / n1h, l = pl % lines, p = pl / lines;
+    const int pl = by_h.div(i), k = i - pl * n1h, p = by_lines.div(pl), l = pl - p * lines;
     const long long li = line0 + l;
     if (li >= nlines) continue;
     const FxLine F = fx_line(emax[1][pl]);
     const int bias = fx_bias<59>(F, sh, -1);
-    const fx2 zk = Z[pl * n1 + k], zn = Z[pl * n1 + (n1 - k) % n1];
+    const fx2 zk = Z[pl * n1 + k], zn = Z[pl * n1 + (k ? n1 - k : 0)];
     const long long row = d.xrow(li) * d.P;
     fx2 A, B;
     A.x = fx_add(zk.x, zn.x); A.y = fx_sub(zk.y, zn.y);
@@ -1417,9 +1417,11 @@ __global__ void __launch_bounds__(512) pass_x_fxg_kernel(double2* __restrict__ s
   }
 }
 
-// Tile [k3][6][cols] of double2, two ping-pong copies.
+// Tile [k3][6][cols] of 16-byte elements, two ping-pong copies.  FIXED: the fixed-point Green step (fx_green_fixed), the tile
+// staying in fixed point between the transforms; otherwise the FP64 one, for every mode of the pass.
+template <bool FIXED>
 __global__ void __launch_bounds__(512) pass_z_fxg_kernel(double2* __restrict__ spec, const fxw* __restrict__ tw, FftPlan plan,
-                                                         Dims d, int cols, GammaParams<double> gp,
+                                                         Dims d, int cols, GammaParams<double> gp, FxGreen G,
                                                          double* __restrict__ partials, SolveState* __restrict__ st, int mode) {
   if (st->done) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1427,44 +1429,74 @@ __global__ void __launch_bounds__(512) pass_z_fxg_kernel(double2* __restrict__ s
   fxw* twl = reinterpret_cast<fxw*>(smem_raw);
   double2* buf = reinterpret_cast<double2*>(twl + n);
   double2* buf2 = buf + n * w6;
+  int* pexp = reinterpret_cast<int*>(buf2 + n * w6);  // [n][cols], FIXED only
   __shared__ double red[32];
-  __shared__ int emax[2][384];
+  __shared__ int emax[2][384], top[64];
   const int k10 = blockIdx.x * cols, k2 = blockIdx.y;
   const LineLayout L{w6, w6, 1, true};
+  const FastDiv by_cols(cols), by_w6(w6);
   for (int i = threadIdx.x; i < n; i += blockDim.x) twl[i] = tw[i];
-  for (int i = threadIdx.x; i < 2 * w6; i += blockDim.x) emax[i / w6][i % w6] = 0;
+  for (int i = threadIdx.x; i < w6; i += blockDim.x) emax[0][i] = emax[1][i] = 0;
+  for (int i = threadIdx.x; i < cols; i += blockDim.x) top[i] = -(1 << 30);
   for (int i = threadIdx.x; i < n * w6; i += blockDim.x) {
-    const int cc = i % cols, rest = i / cols, comp = rest % 6, z = rest / 6;
-    buf[i] = k10 + cc < d.n1h ? spec[comp * d.S + d.row(z, k2) * d.P + k10 + cc] : make_double2(0.0, 0.0);
+    const int z = by_w6.div(i), line = i - z * w6, comp = by_cols.div(line), k1 = k10 + line - comp * cols;
+    buf[i] = k1 < d.n1h ? spec[comp * d.S + d.row(z, k2) * d.P + k1] : make_double2(0.0, 0.0);
   }
   __syncthreads();
   fx_tile_in<60>(buf, emax[0], n, L);
   fx2* r = fx_lines<false>(reinterpret_cast<fx2*>(buf), reinterpret_cast<fx2*>(buf2), twl, plan, L);
   double2* tile = reinterpret_cast<double2*>(r);
   double acc = 0.0, acc2 = 0.0;
-  fx_green_points(n, cols, k10, k2, d, gp, st, mode, nullptr, acc, acc2,
-                  [&](int z, int c, int cc) {
-                    const int i = (z * 6 + c) * cols + cc;
-                    const FxLine F = fx_line(emax[0][c * cols + cc]);
-                    return fx_out(r[i], fx_bias<60>(F, sh, 0), F);
-                  },
-                  [&](int z, int c, int cc, double2 o) { tile[(z * 6 + c) * cols + cc] = o; });
+  if (FIXED) {
+    fx_green_fixed(n, cols, k10, k2, d, gp, G, st, top, acc,
+                   [&](int z, int c, int cc) { return r[(z * 6 + c) * cols + cc]; },
+                   [&](int z, int c, int cc, fx2 o) { r[(z * 6 + c) * cols + cc] = o; },
+                   [&](int c, int cc) { return fx_unit(emax[0][c * cols + cc], sh); },
+                   [&](int z, int cc) -> int& { return pexp[z * cols + cc]; });
+  } else {
+    fx_green_points(n, cols, k10, k2, d, gp, st, mode, nullptr, acc, acc2,
+                    [&](int z, int c, int cc) {
+                      const FxLine F = fx_line(emax[0][c * cols + cc]);
+                      return fx_out(r[(z * 6 + c) * cols + cc], fx_bias<60>(F, sh, 0), F);
+                    },
+                    [&](int z, int c, int cc, double2 o) { tile[(z * 6 + c) * cols + cc] = o; });
+  }
   const int cta = blockIdx.y * gridDim.x + blockIdx.x;
-  if (gp.vprev) {
+  if (!FIXED && gp.vprev) {
     const double s2 = block_sum(acc2, red);
     if (threadIdx.x == 0) gp.cpart[cta] = s2;
     __syncthreads();
   }
-  const double s = block_sum(acc, red);
+  const double s = block_sum(acc, red);  // synchronises the CTA after the Green step's writes
   if (threadIdx.x == 0) partials[cta] = s;
-  fx_tile_in<60>(tile, emax[1], n, L);
+  if (FIXED) {
+    for (int i = threadIdx.x; i < n * w6; i += blockDim.x) {
+      const int z = by_w6.div(i), line = i - z * w6, cc = line - by_cols.div(line) * cols;
+      const int down = top[cc] - pexp[z * cols + cc] + 3;
+      fx2 v = r[i];
+      v.x = fx_sar(v.x, down);
+      v.y = fx_sar(v.y, down);
+      r[i] = v;
+    }
+    __syncthreads();
+  } else {
+    fx_tile_in<60>(tile, emax[1], n, L);
+  }
   fx2* other = reinterpret_cast<fx2*>(tile == buf ? buf2 : buf);
-  r = fx_lines<true>(reinterpret_cast<fx2*>(tile), other, twl, plan, L);
+  r = fx_lines<true>(r, other, twl, plan, L);
   for (int i = threadIdx.x; i < n * w6; i += blockDim.x) {
-    const int cc = i % cols, rest = i / cols, comp = rest % 6, z = rest / 6;
-    if (k10 + cc >= d.n1h) continue;
-    const FxLine F = fx_line(emax[1][comp * cols + cc]);
-    spec[comp * d.S + d.row(z, k2) * d.P + k10 + cc] = fx_out(r[i], fx_bias<60>(F, sh, 0), F);
+    const int z = by_w6.div(i), line = i - z * w6, comp = by_cols.div(line), k1 = k10 + line - comp * cols;
+    if (k1 >= d.n1h) continue;
+    double2 w;
+    if (FIXED) {
+      const FxBack B = fx_back(top[line - comp * cols], G.ef, sh);
+      w = make_double2(fx_to(r[i].x, B.bias), fx_to(r[i].y, B.bias));
+      if (B.far) { w.x *= B.pout; w.y *= B.pout; }
+    } else {
+      const FxLine F = fx_line(emax[1][line]);
+      w = fx_out(r[i], fx_bias<60>(F, sh, 0), F);
+    }
+    spec[comp * d.S + d.row(z, k2) * d.P + k1] = w;
   }
 }
 

@@ -289,6 +289,7 @@ __global__ void pass_x_kernel(typename C<R>::T* __restrict__ spec, R* __restrict
   T* bufb = bufa + 3 * lines * d.n1;
   T* buf = bufa;
   const int n1 = d.n1, n1h = d.n1h;
+  const FastDiv by_n(n1), by_h(n1h), by_lines(lines);
   const long long nlines = (long long)d.n2 * d.n3;
   const long long line0 = (long long)blockIdx.x * lines;
   const bool zero = (flags & PX_ZERO) != 0 || st->restart;
@@ -299,9 +300,8 @@ __global__ void pass_x_kernel(typename C<R>::T* __restrict__ spec, R* __restrict
   if (have_delta) {
     // Hermitian-extend the two half spectra of each component pair into Z = A + i B.
     for (int i = threadIdx.x; i < tot_lines * n1h; i += blockDim.x) {
-      const int k = i % n1h;
-      const int pl = i / n1h;                 // pair * lines + l
-      const int l = pl % lines, p = pl / lines;
+      const int pl = by_h.div(i);             // pair * lines + l
+      const int k = i - pl * n1h, p = by_lines.div(pl), l = pl - p * lines;
       const long long li = line0 + l;
       T z0, z1;
       if (li < nlines) {
@@ -329,7 +329,7 @@ __global__ void pass_x_kernel(typename C<R>::T* __restrict__ spec, R* __restrict
   double dacc = 0.0;
   // state update, sigma = C : eps, repack sigma pairs for the forward transform
   for (int i = threadIdx.x; i < lines * n1; i += blockDim.x) {
-    const int x = i % n1, l = i / n1;
+    const int l = by_n.div(i), x = i - l * n1;
     const long long li = line0 + l;
     if (li >= nlines) continue;
     const long long v = li * n1 + x;
@@ -389,14 +389,13 @@ __global__ void pass_x_kernel(typename C<R>::T* __restrict__ spec, R* __restrict
   buf = fft_lines<false>(buf, buf == bufa ? bufb : bufa, twl, plan, LineLayout{tot_lines, 1, n1, false});
   // split Z = FFT(a + i b) into the half spectra of a and b
   for (int i = threadIdx.x; i < tot_lines * n1h; i += blockDim.x) {
-    const int k = i % n1h;
-    const int pl = i / n1h;
-    const int l = pl % lines, p = pl / lines;
+    const int pl = by_h.div(i);
+    const int k = i - pl * n1h, p = by_lines.div(pl), l = pl - p * lines;
     const long long li = line0 + l;
     if (li >= nlines) continue;
     const T* line = buf + pl * n1;
     const T zk = line[k];
-    const T zn = line[(n1 - k) % n1];
+    const T zn = line[k ? n1 - k : 0];
     T A, B;
     A.x = (R)0.5 * (zk.x + zn.x); A.y = (R)0.5 * (zk.y - zn.y);
     B.x = (R)0.5 * (zk.y + zn.y); B.y = (R)-0.5 * (zk.x - zn.x);
@@ -419,13 +418,14 @@ __global__ void pass_y_kernel(typename C<R>::T* __restrict__ spec, const typenam
   T* buf = twl + d.n2;                       // [n2][cols], plus a ping-pong copy
   T* buf2 = buf + d.n2 * cols;
   const int k10 = blockIdx.x * cols;
+  const FastDiv by_cols(cols);
   const int k3 = blockIdx.y;
   const int c = blockIdx.z;
   for (int i = threadIdx.x; i < d.n2; i += blockDim.x) twl[i] = tw[i];
   T* g = spec + c * d.S + d.row(k3, 0) * d.P + k10;
   const long long ys = d.ystride();
   for (int i = threadIdx.x; i < d.n2 * cols; i += blockDim.x) {
-    const int cc = i % cols, y = i / cols;
+    const int y = by_cols.div(i), cc = i - y * cols;
     T v; v.x = 0; v.y = 0;
     if (k10 + cc < d.n1h) v = g[(long long)y * ys + cc];
     buf[i] = v;
@@ -433,7 +433,7 @@ __global__ void pass_y_kernel(typename C<R>::T* __restrict__ spec, const typenam
   __syncthreads();
   buf = fft_lines<INV>(buf, buf2, twl, plan, LineLayout{cols, cols, 1, true});
   for (int i = threadIdx.x; i < d.n2 * cols; i += blockDim.x) {
-    const int cc = i % cols, y = i / cols;
+    const int y = by_cols.div(i), cc = i - y * cols;
     if (k10 + cc < d.n1h) g[(long long)y * ys + cc] = buf[i];
   }
 }
@@ -505,10 +505,10 @@ __global__ void pass_z_gamma_kernel(typename C<R>::T* __restrict__ spec, const t
   const int k10 = blockIdx.x * cols;
   const int k2 = blockIdx.y;
   const int w6 = 6 * cols;
+  const FastDiv by_cols(cols), by_w6(w6);
   for (int i = threadIdx.x; i < d.n3; i += blockDim.x) twl[i] = tw[i];
   for (int i = threadIdx.x; i < d.n3 * w6; i += blockDim.x) {
-    const int cc = i % cols, rest = i / cols;
-    const int comp = rest % 6, z = rest / 6;
+    const int z = by_w6.div(i), line = i - z * w6, comp = by_cols.div(line), cc = line - comp * cols;
     T v; v.x = 0; v.y = 0;
     if (k10 + cc < d.n1h) v = spec[comp * d.S + d.row(z, k2) * d.P + k10 + cc];
     buf[i] = v;
@@ -521,7 +521,7 @@ __global__ void pass_z_gamma_kernel(typename C<R>::T* __restrict__ spec, const t
   const bool ny2 = ((d.n2 & 1) == 0) && (2 * k2 == d.n2);
   const R b2 = gp.B[1][k2], a2 = gp.A[1][k2];
   for (int i = threadIdx.x; i < d.n3 * cols; i += blockDim.x) {
-    const int cc = i % cols, z = i / cols;
+    const int z = by_cols.div(i), cc = i - z * cols;
     const int k1 = k10 + cc;
     if (k1 >= d.n1h) continue;
     T t[6];
@@ -606,8 +606,7 @@ __global__ void pass_z_gamma_kernel(typename C<R>::T* __restrict__ spec, const t
   if (mode == PZ_RESIDUAL) return;
   buf = fft_lines<true>(buf, other, twl, plan, LineLayout{w6, w6, 1, true});
   for (int i = threadIdx.x; i < d.n3 * w6; i += blockDim.x) {
-    const int cc = i % cols, rest = i / cols;
-    const int comp = rest % 6, z = rest / 6;
+    const int z = by_w6.div(i), line = i - z * w6, comp = by_cols.div(line), cc = line - comp * cols;
     if (k10 + cc < d.n1h) spec[comp * d.S + d.row(z, k2) * d.P + k10 + cc] = buf[i];
   }
 }

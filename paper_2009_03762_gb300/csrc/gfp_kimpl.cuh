@@ -118,7 +118,7 @@ void Passes<R>::pass_x(cudaStream_t s, const LaunchCfg& lc, T* spec, R* eps, con
   const long long nlines = (long long)d.n2 * d.n3;
   const unsigned blocks = (unsigned)((nlines + lc.x_lines - 1) / lc.x_lines);
   const size_t sm = sizeof(T) * (size_t)(d.n1 + 6 * lc.x_lines * d.n1);
-  pass_x_kernel<R><<<blocks, lc.x_threads, sm, s>>>(spec, eps, lam, mu, tw, plan, d, lc.x_lines, flags, pp, st);
+  pass_x_kernel<R><<<blocks, lc.x_threads, sm, s>>>(spec, eps, lam, mu, tw, merge_stages(plan), d, lc.x_lines, flags, pp, st);
 }
 
 template <typename R>
@@ -142,8 +142,8 @@ void Passes<R>::pass_y(cudaStream_t s, const LaunchCfg& lc, bool inverse, T* spe
     default: break;
   }
   const size_t sm = sizeof(T) * (size_t)(d.n2 + 2 * lc.y_cols * d.n2);
-  if (inverse) pass_y_kernel<R, true><<<grid, lc.y_threads, sm, s>>>(spec, tw, plan, d, lc.y_cols, st);
-  else pass_y_kernel<R, false><<<grid, lc.y_threads, sm, s>>>(spec, tw, plan, d, lc.y_cols, st);
+  if (inverse) pass_y_kernel<R, true><<<grid, lc.y_threads, sm, s>>>(spec, tw, merge_stages(plan), d, lc.y_cols, st);
+  else pass_y_kernel<R, false><<<grid, lc.y_threads, sm, s>>>(spec, tw, merge_stages(plan), d, lc.y_cols, st);
 }
 
 template <typename R>
@@ -201,7 +201,7 @@ void Passes<R>::pass_z(cudaStream_t s, const LaunchCfg& lc, T* spec, const W* tw
     default: break;
   }
   const size_t sm = sizeof(T) * (size_t)(d.n3 + 12 * lc.z_cols * d.n3);
-  pass_z_gamma_kernel<R><<<grid, lc.z_threads, sm, s>>>(spec, tw, plan, d, lc.z_cols, gp, partials, st, mode, vsrc);
+  pass_z_gamma_kernel<R><<<grid, lc.z_threads, sm, s>>>(spec, tw, merge_stages(plan), d, lc.z_cols, gp, partials, st, mode, vsrc);
 }
 
 }  // namespace gfp

@@ -392,9 +392,10 @@ __global__ void __launch_bounds__(256) rx_kernel(const float* __restrict__ r, fl
   float2* b = a + nl * n;
   const long long nlines = (long long)d.n2 * d.n3;
   const long long line0 = (long long)blockIdx.x * lines;
+  const FastDiv by_n(n), by_h(NH), by_hp(hp);
   for (int i = threadIdx.x; i < nl * n; i += blockDim.x) {
-    const int e = i % n, q = i / n;
-    const int c = q / hp, p2 = q % hp;
+    const int q = by_n.div(i), e = i - q * n;
+    const int c = by_hp.div(q), p2 = q - c * hp;
     const long long la = line0 + 2 * p2, lb = la + 1;
     float2 z;
     z.x = la < nlines ? r[c * d.N + la * n + e] : 0.f;
@@ -405,11 +406,11 @@ __global__ void __launch_bounds__(256) rx_kernel(const float* __restrict__ r, fl
   LineLayout L{nl, 1, n, false};
   const float2* Z = fft_lines<false>(a, b, tw, plan, L);
   for (int i = threadIdx.x; i < nl * NH; i += blockDim.x) {
-    const int k = i % NH, q = i / NH;
-    const int c = q / hp, p2 = q % hp;
+    const int q = by_h.div(i), k = i - q * NH;
+    const int c = by_hp.div(q), p2 = q - c * hp;
     const long long la = line0 + 2 * p2, lb = la + 1;
     if (la >= nlines) continue;
-    const float2 zk = Z[q * n + k], zn = Z[q * n + (n - k) % n];
+    const float2 zk = Z[q * n + k], zn = Z[q * n + (k ? n - k : 0)];
     float2 A, B;
     A.x = 0.5f * (zk.x + zn.x); A.y = 0.5f * (zk.y - zn.y);
     B.x = 0.5f * (zk.y + zn.y); B.y = -0.5f * (zk.x - zn.x);
@@ -433,8 +434,9 @@ __global__ void __launch_bounds__(256) rz_kernel(float2* __restrict__ v, const f
   const int k10 = blockIdx.x * cols, k2 = blockIdx.y, c = blockIdx.z;
   float2* g = v + c * d.S + d.row(0, k2) * d.P;
   const long long zs = d.zstride();
+  const FastDiv by_cols(cols);
   for (int i = threadIdx.x; i < cols * n; i += blockDim.x) {
-    const int l = i % cols, e = i / cols;
+    const int e = by_cols.div(i), l = i - e * cols;
     float2 z; z.x = 0.f; z.y = 0.f;
     if (k10 + l < d.n1h) z = g[e * zs + k10 + l];
     a[l * ls + e] = z;
@@ -445,7 +447,7 @@ __global__ void __launch_bounds__(256) rz_kernel(float2* __restrict__ v, const f
   float2 p2; p2.x = 1.f; p2.y = 0.f;
   if (ph2) p2 = ph2[k2];
   for (int i = threadIdx.x; i < cols * n; i += blockDim.x) {
-    const int l = i % cols, e = i / cols;
+    const int e = by_cols.div(i), l = i - e * cols;
     const int k1 = k10 + l;
     if (k1 >= d.n1h) continue;
     float2 z = Z[l * ls + e];
