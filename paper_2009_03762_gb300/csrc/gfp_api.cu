@@ -1012,11 +1012,11 @@ int solve_fp64(gfp_grid g, const gfp_scheme* sc, const double E[6], double tol, 
   // the mean stress of the final strain by a compensated real-space sum (the k = 0 value of the
   // transform rounds at about 1e-16 of it)
   if (g->st_host->done != DONE_TIMEOUT) {
-    const int mb = 512;
+    const int mb = (int)std::max<long long>(1, std::min<long long>(608, g->d.N / 512));
     double* mpart = g->scratch;  // 8 K doubles: 12 per block
     mean_stress64_kernel<<<mb, 256, 0, g->stream>>>(g->eps, g->lam, g->mu, g->estar_on ? g->estar : nullptr,
                                                     g->d.N, mpart);
-    mean_stress64_final_kernel<<<1, 32, 0, g->stream>>>(mpart, mb, g->st);
+    mean_stress64_final_kernel<<<1, 192, 0, g->stream>>>(mpart, mb, g->st);
     g->launches += 2;
     GFP_CU(cudaGetLastError());
     GFP_CU(cudaMemcpyAsync(g->st_host->T0, g->st->T0, sizeof(double) * 6, cudaMemcpyDeviceToHost, g->stream));

@@ -297,61 +297,90 @@ __global__ void __launch_bounds__(kResTX * kResTY) residual64_afd_kernel(const d
   }
 }
 
-// Mean stress of an FP64 strain field with compensated summation: sigma = C : (eps - estar) per voxel,
-// summed per thread and per CTA in Neumaier's form (running sum plus the accumulated rounding
-// errors), per-CTA (sum, compensation) pairs into part[12 b + 2 c], then combined in a fixed order by
-// mean_stress64_final_kernel.  The sum the transform forms at k = 0 rounds at about 1e-16 of the mean
-// stress, which is the size of the change one voxel's modulus makes in the effective stiffness of a
-// 128^3 cell; this sum keeps the rounding well below it.
-__device__ __forceinline__ void neumaier_add(double& s, double& c, double x) {
-  const double t = s + x;
-  c += fabs(s) >= fabs(x) ? (s - t) + x : (x - t) + s;
-  s = t;
+// Mean stress of an FP64 strain field with compensated summation: sigma = C : (eps - estar) per voxel.  A thread adds the
+// stresses of four voxels in FP64 (their rounding, 2^-53 of four terms, averages out over N / 4 groups to below 1e-18 of
+// the mean at 64^3) and gathers these sums with their rounding errors (TwoSum); pairs (sum, errors) are combined the same way
+// by a warp per component, per CTA into part[12 b + 2 c] and by mean_stress64_final_kernel in a fixed order.  The sum the transform
+// forms at k = 0 rounds at about 1e-16 of the mean stress, which is the size of the change one voxel's modulus makes in
+// the effective stiffness of a 128^3 cell; this sum keeps the rounding well below it.  FP64 operations bound it (31 a voxel;
+// one compensated addition per voxel took 55) with the serial ends before: 256^3 2.16 + 0.16 ->
+// 0.82 + 0.01 ms, 32^3 87 + 152 -> 13 + 5 us.
+struct SumErr {
+  double s, e;
+  __device__ __forceinline__ void add(double x) {
+    const double t = s + x, v = t - s;
+    e += (s - (t - v)) + (x - v);
+    s = t;
+  }
+  __device__ __forceinline__ void add(const SumErr& o) {
+    add(o.s);
+    e += o.e;
+  }
+};
+__device__ __forceinline__ void warp_sum(SumErr& a) {
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) {
+    SumErr o;
+    o.s = __shfl_down_sync(0xffffffffu, a.s, off);
+    o.e = __shfl_down_sync(0xffffffffu, a.e, off);
+    a.add(o);
+  }
 }
 
 __global__ void __launch_bounds__(256) mean_stress64_kernel(const double* __restrict__ eps, const double* __restrict__ lam,
                                                           const double* __restrict__ mu, const double* __restrict__ estar,
                                                           long long N, double* __restrict__ part) {
-  __shared__ double sh[256][12];
-  double s[6] = {0, 0, 0, 0, 0, 0}, cp[6] = {0, 0, 0, 0, 0, 0};
-  for (long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x; v < N; v += (long long)gridDim.x * blockDim.x) {
-    double e[6];
+  __shared__ SumErr sh[6][256];
+  SumErr a[6] = {};
+  const long long step = (long long)gridDim.x * blockDim.x;
+  for (long long v0 = blockIdx.x * (long long)blockDim.x + threadIdx.x; v0 < N; v0 += 4 * step) {
+    double x[6] = {0, 0, 0, 0, 0, 0};
 #pragma unroll
-    for (int c = 0; c < 6; ++c) e[c] = eps[c * N + v] - (estar ? estar[c * N + v] : 0.0);
-    const double m2 = 2.0 * mu[v], ltr = lam[v] * (e[0] + e[1] + e[2]);
-    neumaier_add(s[0], cp[0], m2 * e[0] + ltr);
-    neumaier_add(s[1], cp[1], m2 * e[1] + ltr);
-    neumaier_add(s[2], cp[2], m2 * e[2] + ltr);
-    neumaier_add(s[3], cp[3], m2 * e[3]);
-    neumaier_add(s[4], cp[4], m2 * e[4]);
-    neumaier_add(s[5], cp[5], m2 * e[5]);
+    for (int q = 0; q < 4; ++q) {
+      const long long v = v0 + q * step;
+      if (v >= N) continue;
+      double e[6];
+#pragma unroll
+      for (int c = 0; c < 6; ++c) e[c] = eps[c * N + v];
+      if (estar) {
+#pragma unroll
+        for (int c = 0; c < 6; ++c) e[c] -= estar[c * N + v];
+      }
+      const double m2 = 2.0 * mu[v], ltr = lam[v] * (e[0] + e[1] + e[2]);
+#pragma unroll
+      for (int c = 0; c < 6; ++c) x[c] += c < 3 ? m2 * e[c] + ltr : m2 * e[c];
+    }
+#pragma unroll
+    for (int c = 0; c < 6; ++c) a[c].add(x[c]);
   }
 #pragma unroll
-  for (int c = 0; c < 6; ++c) { sh[threadIdx.x][2 * c] = s[c]; sh[threadIdx.x][2 * c + 1] = cp[c]; }
+  for (int c = 0; c < 6; ++c) sh[c][threadIdx.x] = a[c];
   __syncthreads();
-  if (threadIdx.x < 6) {
-    const int c = threadIdx.x;
-    double ss = 0.0, cc = 0.0;
-    for (int i = 0; i < (int)blockDim.x; ++i) {
-      neumaier_add(ss, cc, sh[i][2 * c]);
-      cc += sh[i][2 * c + 1];
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (w < 6) {  // a warp per component: 13 additions deep, where shuffles of all warps would add 6 x 5 times per warp
+    SumErr t = sh[w][lane];
+#pragma unroll
+    for (int k = 1; k < 8; ++k) t.add(sh[w][lane + 32 * k]);
+    warp_sum(t);
+    if (lane == 0) {
+      part[12 * blockIdx.x + 2 * w] = t.s;
+      part[12 * blockIdx.x + 2 * w + 1] = t.e;
     }
-    part[12 * blockIdx.x + 2 * c] = ss;
-    part[12 * blockIdx.x + 2 * c + 1] = cc;
   }
 }
 
-// Fixed-order combination of the per-CTA pairs: st->T0[c] = sum sigma_c (the transform at k = 0).
+// Fixed-order combination of the per-CTA pairs, a warp per component: st->T0[c] = sum sigma_c (the transform at k = 0).
 __global__ void mean_stress64_final_kernel(const double* __restrict__ part, int nb, SolveState* st) {
-  if (threadIdx.x < 6) {
-    const int c = threadIdx.x;
-    double ss = 0.0, cc = 0.0;
-    for (int b = 0; b < nb; ++b) {
-      neumaier_add(ss, cc, part[12 * b + 2 * c]);
-      cc += part[12 * b + 2 * c + 1];
-    }
-    st->T0[c] = ss + cc;
+  const int c = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  SumErr a = {0.0, 0.0};
+  for (int b = lane; b < nb; b += 32) {
+    SumErr o;
+    o.s = part[12 * b + 2 * c];
+    o.e = part[12 * b + 2 * c + 1];
+    a.add(o);
   }
+  warp_sum(a);
+  if (lane == 0) st->T0[c] = a.s + a.e;
 }
 
 // Sum of the per-CTA residual sums in a fixed order: st->T0 = sum sigma (the transform at k = 0) and
