@@ -915,6 +915,16 @@ int ensure_hist(gfp_grid g, int cap) {
   return GFP_OK;
 }
 
+// Iterations to launch before the next look at the device state: twice as many as last time, up to 64, but no more than the
+// solve should still need at the rate at which the last `steps` iterations brought eta from eta0 to eta1 (and one more; kernels
+// launched beyond convergence do nothing but still take 2 us each).
+int next_chunk(int chunk, double eta0, double eta1, int steps, double tol) {
+  const int twice = std::min(2 * chunk, 64);
+  if (!(tol > 0.0) || steps < 1 || !(eta1 > tol) || !(eta1 < eta0) || !std::isfinite(eta0)) return twice;
+  const double need = std::ceil(std::log(tol / eta1) / std::log(eta1 / eta0) * steps) + 1.0;
+  return need < twice ? std::max(1, (int)need) : twice;
+}
+
 // F and HC average the Green operator over Hermitian partners on the Nyquist planes, which only even axes have.
 int nyquist_average(int op, const Dims& d) {
   return (op == OP_F || op == OP_HC) && (d.n1 % 2 == 0 || d.n2 % 2 == 0 || d.n3 % 2 == 0) ? 1 : 0;
@@ -998,6 +1008,7 @@ int solve_fp64(gfp_grid g, const gfp_scheme* sc, const double E[6], double tol, 
   GFP_CU(cudaMemcpyAsync(g->st, g->st_host, sizeof(SolveState), cudaMemcpyHostToDevice, g->stream));
   int launched = 0;
   int chunk = 2;
+  double eta0 = INFINITY;
   const int budget = maxit - start_it;
   while (launched < budget) {
     const int nb = std::min(chunk, budget - launched);
@@ -1007,7 +1018,9 @@ int solve_fp64(gfp_grid g, const gfp_scheme* sc, const double E[6], double tol, 
     GFP_CU(cudaMemcpyAsync(g->st_host, g->st, sizeof(SolveState), cudaMemcpyDeviceToHost, g->stream));
     GFP_CU(cudaStreamSynchronize(g->stream));
     if (g->st_host->done) break;
-    chunk = std::min(chunk * 2, 64);
+    const double eta1 = rule1 ? g->st_host->crit : g->st_host->eta;
+    chunk = next_chunk(chunk, eta0, eta1, nb, tol);
+    eta0 = eta1;
   }
   // the mean stress of the final strain by a compensated real-space sum (the k = 0 value of the
   // transform rounds at about 1e-16 of it)
@@ -1247,6 +1260,7 @@ int solve_mixed(gfp_grid g, const gfp_scheme* sc, const double E[6], double tol,
     *g->st_in_host = si;
     GFP_CU(cudaMemcpyAsync(g->st_in, g->st_in_host, sizeof(SolveState), cudaMemcpyHostToDevice, g->stream));
     int launched = 0, chunk = 4;
+    double eta0 = INFINITY;
     while (launched < si.maxit) {
       const int nb = std::min(chunk, si.maxit - launched);
       for (int b = 0; b < nb; ++b) inner_iteration32(g, gp32, (launched + b) == 0 ? PX_ZERO : PX_DELTA);
@@ -1255,7 +1269,8 @@ int solve_mixed(gfp_grid g, const gfp_scheme* sc, const double E[6], double tol,
       GFP_CU(cudaMemcpyAsync(g->st_in_host, g->st_in, sizeof(SolveState), cudaMemcpyDeviceToHost, g->stream));
       GFP_CU(cudaStreamSynchronize(g->stream));
       if (g->st_in_host->done) break;
-      chunk = std::min(chunk * 2, 64);
+      chunk = next_chunk(chunk, eta0, g->st_in_host->eta, nb, si.tol);
+      eta0 = g->st_in_host->eta;
     }
     inner_total += g->st_in_host->it;
     if (g->st_in_host->done == 3) { status = GFP_ERR_DIVERGED; break; }
@@ -1418,6 +1433,7 @@ int solve_dgo(gfp_grid g, const gfp_scheme* sc, const double E[6], double tol, i
   GFP_CU(cudaMemcpyAsync(g->st, g->st_host, sizeof(SolveState), cudaMemcpyHostToDevice, g->stream));
   const int np = d.n2 * d.n3;
   int launched = 0, chunk = 2;
+  double eta0 = INFINITY;
   while (launched < maxit + 1) {
     const int nb = std::min(chunk, maxit + 1 - launched);
     for (int b = 0; b < nb; ++b) {
@@ -1437,7 +1453,8 @@ int solve_dgo(gfp_grid g, const gfp_scheme* sc, const double E[6], double tol, i
     GFP_CU(cudaMemcpyAsync(g->st_host, g->st, sizeof(SolveState), cudaMemcpyDeviceToHost, g->stream));
     GFP_CU(cudaStreamSynchronize(g->stream));
     if (g->st_host->done) break;
-    chunk = std::min(chunk * 2, 64);
+    chunk = next_chunk(chunk, eta0, g->st_host->eta, nb, tol);
+    eta0 = g->st_host->eta;
   }
   const SolveState s = *g->st_host;
   // mean stress of the final strain
@@ -2037,6 +2054,7 @@ int gfp_solve_noalloc(int n1, int n2, int n3, double h, const double* lambda, co
   GFP_CU(cudaMemcpyAsync(st, &sh, sizeof(SolveState), cudaMemcpyHostToDevice, stream));
   GFP_CU(cudaStreamSynchronize(stream));
   int launched = 0, chunk = 2;
+  double eta0 = INFINITY;
   while (launched < maxit) {
     const int nb = std::min(chunk, maxit - launched);
     for (int b = 0; b < nb; ++b) {
@@ -2052,7 +2070,8 @@ int gfp_solve_noalloc(int n1, int n2, int n3, double h, const double* lambda, co
     GFP_CU(cudaMemcpyAsync(&sh, st, sizeof(SolveState), cudaMemcpyDeviceToHost, stream));
     GFP_CU(cudaStreamSynchronize(stream));
     if (sh.done) break;
-    chunk = std::min(chunk * 2, 64);
+    chunk = next_chunk(chunk, eta0, sh.eta, nb, tol);
+    eta0 = sh.eta;
   }
   int status = GFP_OK;
   if (sh.done == 2 || sh.done == 0) status = GFP_ERR_NOT_CONVERGED;
