@@ -193,8 +193,14 @@ __global__ void corr_mean_partial_kernel(const float* __restrict__ corr, long lo
   __shared__ double sh[6][256];
   double acc[6] = {0, 0, 0, 0, 0, 0};
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x) {
+    float f[6];
+    double w[6];
 #pragma unroll
-    for (int c = 0; c < 6; ++c) acc[c] += (double)corr[c * N + i];
+    for (int c = 0; c < 6; ++c) f[c] = corr[c * N + i];
+#pragma unroll
+    for (int c = 0; c < 6; ++c) w[c] = widen(f[c]);
+#pragma unroll
+    for (int c = 0; c < 6; ++c) acc[c] += w[c];
   }
 #pragma unroll
   for (int c = 0; c < 6; ++c) sh[c][threadIdx.x] = acc[c];
@@ -207,15 +213,17 @@ __global__ void corr_mean_partial_kernel(const float* __restrict__ corr, long lo
   if (threadIdx.x < 6) part[blockIdx.x * 6 + threadIdx.x] = sh[threadIdx.x][0];
 }
 
-// stage 2: one block, fixed order
+// stage 2: a warp per component, fixed order (one thread per component took 57 us for 1024 blocks: a chain of loads)
 __global__ void corr_mean_final_kernel(const double* __restrict__ part, int nb, long long N, double* __restrict__ mean,
                                        const SolveState* gate) {
   if (gate && gate->done == 2) return;
-  if (threadIdx.x < 6) {
-    double s = 0.0;
-    for (int b = 0; b < nb; ++b) s += part[b * 6 + threadIdx.x];
-    mean[threadIdx.x] = s / (double)N;
-  }
+  const int c = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  double s = 0.0;
+#pragma unroll 8
+  for (int b = lane; b < nb; b += 32) s += part[b * 6 + c];
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) s += __shfl_down_sync(0xffffffffu, s, off);
+  if (lane == 0) mean[c] = s / (double)N;
 }
 
 
@@ -1140,6 +1148,9 @@ GammaParams<R> gamma_params(gfp_grid g, int op, const R* const* A, const R* cons
   return gp;
 }
 
+// Blocks of the passes over the FP32 correction: one wave, four per SM (1024 left a second wave one third full).
+inline int corr_blocks(const Dims& d) { return (int)std::min<long long>(608, (d.N + 255) / 256); }
+
 // Real-space FP64 outer pass (gfp_outer.cuh) on explicit buffers, for single and batched solves:
 // eps += corr - mean(corr) (if corr), r = D^b C : (eps - estar), the FP64 residual and mean stress
 // into st (reduce_eta decides convergence).  r (FP32 [3][N]) goes to rbuf.  Every kernel is a no-op
@@ -1148,16 +1159,21 @@ void outer_pass64(cudaStream_t s, const Dims& d, double h, int op, double* eps, 
                   const double* estar, const float* corr, const double* cmean, float* rbuf, double* rpart,
                   double* partials, SolveState* st, long long& launches) {
   if (corr) {
-    const int cvb = (int)std::min<long long>(1024, (d.N + 255) / 256);
+    const int cvb = corr_blocks(d);
     apply_corr64_kernel<<<cvb, 256, 0, s>>>(eps, corr, cmean, d.N, st);
     ++launches;
   }
   const dim3 grid = res64_grid(d);
   const double inv_h = 1.0 / h;
+  auto residual = [&](auto sten, auto est) {
+    constexpr int S = decltype(sten)::value;
+    residual_fx_kernel<S, decltype(est)::value><<<grid, ResHalo<S>::NT, 0, s>>>(eps, lam, mu, estar, d, inv_h, rbuf, rpart, st);
+  };
+  auto stencil = [&](auto st_) { estar ? residual(st_, std::true_type{}) : residual(st_, std::false_type{}); };
   switch (res_stencil(op)) {
-    case RS_CD: residual64_kernel<RS_CD><<<grid, kResTX * kResTY, 0, s>>>(eps, lam, mu, estar, d, inv_h, rbuf, rpart, st); break;
-    case RS_ACD: residual64_kernel<RS_ACD><<<grid, kResTX * kResTY, 0, s>>>(eps, lam, mu, estar, d, inv_h, rbuf, rpart, st); break;
-    default: residual64_afd_kernel<<<grid, kResTX * kResTY, 0, s>>>(eps, lam, mu, estar, d, inv_h, rbuf, rpart, st); break;
+    case RS_CD: stencil(std::integral_constant<int, RS_CD>{}); break;
+    case RS_ACD: stencil(std::integral_constant<int, RS_ACD>{}); break;
+    default: stencil(std::integral_constant<int, RS_AFD>{}); break;
   }
   res64_sum_kernel<<<1, 256, 0, s>>>(rpart, res64_blocks(d), d.N, st, partials);
   launch_reduce_eta(s, partials, 1, st, nullptr, 0);
@@ -1218,7 +1234,7 @@ int solve_mixed(gfp_grid g, const gfp_scheme* sc, const double E[6], double tol,
   rc = ensure_tables(g, sc->op);
   if (rc) return rc;
   const Dims& d = g->d;
-  const int cvb = (int)std::min<long long>(1024, (d.N + 255) / 256);
+  const int cvb = corr_blocks(d);
   if (!g->lam32_valid) {
     to_float_kernel<<<cvb, 256, 0, g->stream>>>(g->lam, g->lam32, d.N);
     to_float_kernel<<<cvb, 256, 0, g->stream>>>(g->mu, g->mu32, d.N);
@@ -1276,7 +1292,7 @@ int solve_mixed(gfp_grid g, const gfp_scheme* sc, const double E[6], double tol,
     if (g->st_in_host->done == 3) { status = GFP_ERR_DIVERGED; break; }
     if (g->st_in_host->done == DONE_TIMEOUT) { status = GFP_ERR_DEVICE_TIMEOUT; break; }
     corr_mean_partial_kernel<<<cvb, 256, 0, g->stream>>>(g->eps32, d.N, g->cpart, nullptr);
-    corr_mean_final_kernel<<<1, 32, 0, g->stream>>>(g->cpart, cvb, d.N, g->cmean, nullptr);
+    corr_mean_final_kernel<<<1, 192, 0, g->stream>>>(g->cpart, cvb, d.N, g->cmean, nullptr);
     g->launches += 2;
     // the next outer pass re-arms the FP64 state (it counts outer passes; never stops on maxit)
     g->st_host->done = 0;
@@ -2322,7 +2338,7 @@ void slot_window(BatchSlot& s, int op, const GammaParams<float>& gp32, const Bat
   gfp_grid g = s.g;
   const Dims& d = g->d;
   cudaStream_t st = s.stream;
-  const int cvb = (int)std::min<long long>(1024, (d.N + 255) / 256);
+  const int cvb = corr_blocks(d);
   batch_init_kernel<<<(int)std::min<long long>(4096, (6 * d.N + 255) / 256), 256, 0, st>>>(
       s.eps, s.eps32, d.N, s.load, s.st, s.st_in, s.acc, s.cmean, windows, ctl);
   batch_gate_kernel<<<1, 32, 0, st>>>(s.st, s.st_in, window);
@@ -2342,7 +2358,7 @@ void slot_window(BatchSlot& s, int op, const GammaParams<float>& gp32, const Bat
     Passes<float>::pass_y(st, s.lc32, true, spec32, g->tw32[1], s.lc32.plan[1], d, s.st_in);
   }
   corr_mean_partial_kernel<<<cvb, 256, 0, st>>>(s.eps32, d.N, s.cpart, s.st_in);
-  corr_mean_final_kernel<<<1, 32, 0, st>>>(s.cpart, cvb, d.N, s.cmean, s.st_in);
+  corr_mean_final_kernel<<<1, 192, 0, st>>>(s.cpart, cvb, d.N, s.cmean, s.st_in);
 }
 
 }  // namespace

@@ -18,13 +18,14 @@
 // FP64 transform, and the source comes from an FP32 transform of r: v is stored in FP32 and r carries
 // its own scale, so the FP32 transform keeps v's relative accuracy.
 #pragma once
-#include "gfp_kernels.cuh"
+#include "gfp_fxnum.cuh"
 
 namespace gfp {
 
 enum { RS_CD = 0, RS_ACD = 1, RS_AFD = 2 };
 
-// Refinement step of the FP64 strain: eps += corr - mean(corr) (skipped while `gate` is done).
+// Refinement step of the FP64 strain: eps += corr - mean(corr) (skipped while `gate` is done).  Bound by HBM (120 B a
+// voxel) once the conversions left the FP64 pipe (2 a clock and SM): 512^3 4.89 -> 3.51 ms.
 __global__ void apply_corr64_kernel(double* __restrict__ eps, const float* __restrict__ corr,
                                     const double* __restrict__ cmean, long long N, const SolveState* gate) {
   if (gate && gate->done) return;
@@ -32,268 +33,216 @@ __global__ void apply_corr64_kernel(double* __restrict__ eps, const float* __res
 #pragma unroll
   for (int c = 0; c < 6; ++c) cm[c] = cmean[c];
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x) {
+    float f[6];
+    double w[6];
 #pragma unroll
-    for (int c = 0; c < 6; ++c) eps[c * N + i] += (double)corr[c * N + i] - cm[c];
+    for (int c = 0; c < 6; ++c) f[c] = corr[c * N + i];
+#pragma unroll
+    for (int c = 0; c < 6; ++c) w[c] = widen(f[c]);
+#pragma unroll
+    for (int c = 0; c < 6; ++c) eps[c * N + i] += w[c] - cm[c];
   }
 }
 
 // Tile of the real-space residual: RX x RY columns marched over RZ planes, one voxel of halo on each
-// side (periodic).  A CTA of RX RY threads keeps the stress of three consecutive halo planes in
+// side (periodic).  A CTA has a thread per point of a halo plane and keeps one plane's stress in
 // shared memory.
 constexpr int kResTX = 32, kResTY = 8, kResTZ = 16;
 
 // sigma = C : (eps - estar) (FP64), r = D^b sigma rounded to FP32 into rout [3][N], and per CTA the
 // FP64 sums part[8 b + 0] = sum |r|^2 and part[8 b + 1 + c] = sum sigma_c over the CTA's voxels.
-template <int S>
-__global__ void __launch_bounds__(kResTX * kResTY) residual64_kernel(const double* __restrict__ eps,
-                                                                     const double* __restrict__ lam,
+//
+// Each plane is visited once and its part of the next plane's r carried on (M).  Averaged stencils (ACD; AHC and AFB/R): in a
+// thread's 2x2 window on plane z, with g_ab = f(x + a, y + b, z), a, b in {-1, 1} (ACD) or {0, 1} (AFD),
+//   Qx f = (g10 - g00) + (g11 - g01),  Qy f = (g01 - g00) + (g11 - g10),  P f = g00 + g01 + g10 + g11,
+// and D_x f(z) = Qx f(z + lo) + Qx f(z + 1), D_y f likewise, D_z f(z) = P f(z + 1) - P f(z + lo), lo = -1 (ACD) or 0
+// (AFD).  So r_1(z) = M_1(z + lo) + S_1(z + 1) with S_1 = Qx s11 + Qy s12 + P s13 and M_1 = Qx s11 + Qy s12 - P s13 (and
+// likewise r_2 from s12, s22, s23 and r_3 from s13, s23, s33).  CD: r_1(z) = [dx s11 + dy s12](z) - s13(z - 1) + s13(z + 1).
+//
+// The stress is formed in FP64 (2 operations per clock and SM) and added in integers: 58 bits below the largest stress the
+// CTA has met, rounded, so that the 24 terms of a sum and the 16 planes of a mean stay in range; the error of a term, 2^-59 of
+// that stress, is below the rounding of stresses down to 1/64 of it.  The exponent only rises: what is carried is shifted where a plane
+// raises it.  With sums in FP64 (18 to 60 operations a voxel) against this: AFB/R 256^3 2.16 -> 0.76 ms, 512^3 17.1 -> 5.96;
+// ACD 512^3 15.1 (FP64 stress sums) -> 6.4; CD 512^3 13.0 -> 6.8.
+template <int S> struct ResHalo {
+  static constexpr int LO = S == RS_AFD ? 0 : 1, HX = kResTX + 1 + LO, HY = kResTY + 1 + LO;
+  static constexpr int NT = (HX * HY + 31) / 32 * 32;  // a thread per point of the tile with its halo
+};
+template <int S, bool EST>
+__global__ void __launch_bounds__(ResHalo<S>::NT) residual_fx_kernel(const double* __restrict__ eps, const double* __restrict__ lam,
                                                                      const double* __restrict__ mu,
-                                                                     const double* __restrict__ estar, Dims d,
-                                                                     double inv_h, float* __restrict__ rout,
-                                                                     double* __restrict__ part,
+                                                                     const double* __restrict__ estar, Dims d, double inv_h,
+                                                                     float* __restrict__ rout, double* __restrict__ part,
                                                                      const SolveState* gate) {
   if (gate && gate->done) return;
-  constexpr int HX = kResTX + 2, HY = kResTY + 2, NT = kResTX * kResTY;
-  __shared__ double sg[3][6][HY][HX];
-  __shared__ double red[NT / 32][8];
+  constexpr int LO = ResHalo<S>::LO, HX = ResHalo<S>::HX, HY = ResHalo<S>::HY, NO = kResTX * kResTY;
+  __shared__ long long sg[6][HY * HX];
+  __shared__ double red[NO / 32][8];
+  __shared__ int top[2];  // largest high word of the stress, by plane parity
   const int n1 = d.n1, n2 = d.n2, n3 = d.n3;
   const long long N = d.N;
-  const int x0 = blockIdx.x * kResTX, y0 = blockIdx.y * kResTY, z0 = blockIdx.z * kResTZ;
-  const int tx = threadIdx.x % kResTX, ty = threadIdx.x / kResTX;
-  const bool col_ok = (x0 + tx < n1) && (y0 + ty < n2);
-  const int nz = min(kResTZ, n3 - z0);
-  double ss[6] = {0, 0, 0, 0, 0, 0};
-  float rr = 0.f;  // eta needs relative accuracy only; r itself is FP64
-  // the averaged forward differences need the halo on the high side only
-  constexpr int LO = S == RS_AFD ? 1 : 0, RW = HX - LO, RH = HY - LO;
-#pragma unroll 1
-  for (int p = S == RS_AFD ? 1 : 0; p < nz + 2; ++p) {
-    const int zw = ((z0 - 1 + p) % n3 + n3) % n3;
-    const int slot = p % 3;
-    for (int i = threadIdx.x; i < RW * RH; i += NT) {
-      const int hx = LO + i % RW, hy = LO + i / RW;
-      const int xg = ((x0 - 1 + hx) % n1 + n1) % n1;
-      const int yg = ((y0 - 1 + hy) % n2 + n2) % n2;
-      const long long v = ((long long)zw * n2 + yg) * n1 + xg;
-      double e[6];
-#pragma unroll
-      for (int c = 0; c < 6; ++c) e[c] = eps[c * N + v];
-      if (estar) {
-#pragma unroll
-        for (int c = 0; c < 6; ++c) e[c] -= estar[c * N + v];
-      }
-      const double m2 = 2.0 * mu[v], ltr = lam[v] * (e[0] + e[1] + e[2]);
-      double sgm[6];
-      sgm[0] = m2 * e[0] + ltr;
-      sgm[1] = m2 * e[1] + ltr;
-      sgm[2] = m2 * e[2] + ltr;
-      sgm[3] = m2 * e[3];
-      sgm[4] = m2 * e[4];
-      sgm[5] = m2 * e[5];
-#pragma unroll
-      for (int c = 0; c < 6; ++c) sg[slot][c][hy][hx] = sgm[c];
-      const bool own = hx >= 1 && hx <= kResTX && hy >= 1 && hy <= kResTY && p >= 1 && p <= nz &&
-                       x0 - 1 + hx < n1 && y0 - 1 + hy < n2;
-      if (own) {
-#pragma unroll
-        for (int c = 0; c < 6; ++c) ss[c] += sgm[c];
-      }
+  const int x0 = blockIdx.x * kResTX, y0 = blockIdx.y * kResTY, z0 = blockIdx.z * kResTZ, t0 = threadIdx.x;
+  // the point this thread loads, and the one it writes: the first NO threads' points are the tile itself, the others' its halo
+  int hx, hy;
+  if (t0 < NO) {
+    hx = LO + t0 % kResTX;
+    hy = LO + t0 / kResTX;
+  } else {
+    const int i = t0 - NO, rows = HY - kResTY;  // whole rows below (LO) and above, then the columns beside the tile
+    if (i < rows * HX) {
+      hx = i % HX;
+      hy = LO && i < HX ? 0 : HY - 1;
+    } else {
+      const int k = i - rows * HX;
+      hx = LO && k % 2 == 0 ? 0 : HX - 1;
+      hy = LO + k / (1 + LO);
     }
-    __syncthreads();
-    if (p >= 2 && col_ok) {
-      // outputs on plane p - 1 (z = z0 + p - 2); its neighbours below and above are planes p - 2, p
-      const int sl[3] = {(p - 2) % 3, (p - 1) % 3, p % 3};
-      const int hx = tx + 1, hy = ty + 1;
-      // stress component c at offset (dx, dy, dz) from the output voxel
-      auto f = [&](int c, int dx, int dy, int dz) -> double { return sg[sl[dz + 1]][c][hy + dy][hx + dx]; };
-      // component c at offsets (oj, oa, ob) along (e_j, e_a, e_b), (a, b) the axes after j cyclically
-      auto at = [&](int c, int jj, int oj, int oa, int ob) -> double {
-        int o[3];
-        o[jj] = oj;
-        o[(jj + 1) % 3] = oa;
-        o[(jj + 2) % 3] = ob;
-        return f(c, o[0], o[1], o[2]);
-      };
-      const double sc = (S == RS_CD ? 0.5 : (S == RS_ACD ? 0.125 : 0.25)) * inv_h;
-      double r1, r2, r3;
-      if (S == RS_AFD) {
-        // over the unit cube, with the pair sums along the third axis shared by a component's two
-        // derivatives: D_u f = [p(1,0) + p(1,1)] - [p(0,0) + p(0,1)], p(a,b) = f(a,b,0) + f(a,b,1)
-        auto one = [&](int c, int u) -> double {  // single derivative along axis u
-          const double hi = (at(c, u, 1, 0, 0) + at(c, u, 1, 0, 1)) + (at(c, u, 1, 1, 0) + at(c, u, 1, 1, 1));
-          const double lo = (at(c, u, 0, 0, 0) + at(c, u, 0, 0, 1)) + (at(c, u, 0, 1, 0) + at(c, u, 0, 1, 1));
-          return hi - lo;
-        };
-        // two derivatives along u and v = (u + 1) % 3 of component c, sharing the sums along w
-        auto two = [&](int c, int u, double& du, double& dv) {
-          double q[2][2];
-#pragma unroll
-          for (int a = 0; a <= 1; ++a)
-#pragma unroll
-            for (int b = 0; b <= 1; ++b) q[a][b] = at(c, u, a, b, 0) + at(c, u, a, b, 1);
-          du = (q[1][0] + q[1][1]) - (q[0][0] + q[0][1]);
-          dv = (q[0][1] + q[1][1]) - (q[0][0] + q[1][0]);
-        };
-        double d12x, d12y, d23y, d23z, d13z, d13x;
-        two(5, 0, d12x, d12y);  // sigma_12: D_1, D_2
-        two(3, 1, d23y, d23z);  // sigma_23: D_2, D_3
-        two(4, 2, d13z, d13x);  // sigma_13: D_3, D_1
-        r1 = sc * (one(0, 0) + d12y + d13z);
-        r2 = sc * (d12x + one(1, 1) + d23z);
-        r3 = sc * (d13x + d23y + one(2, 2));
-      } else {
-      // D_j of component c, unscaled
-      auto D = [&](int c, int jj) -> double {
-        double acc = 0.0;
-        if (S == RS_CD) {
-          acc = at(c, jj, 1, 0, 0) - at(c, jj, -1, 0, 0);
-        } else if (S == RS_ACD) {
-#pragma unroll
-          for (int sa = -1; sa <= 1; sa += 2)
-#pragma unroll
-            for (int sb = -1; sb <= 1; sb += 2) acc += at(c, jj, 1, sa, sb) - at(c, jj, -1, sa, sb);
-        } else {
-#pragma unroll
-          for (int oa = 0; oa <= 1; ++oa)
-#pragma unroll
-            for (int ob = 0; ob <= 1; ++ob) acc += at(c, jj, 1, oa, ob) - at(c, jj, 0, oa, ob);
-        }
-        return acc;
-      };
-      // components (11, 22, 33, 23, 13, 12) = (0, 1, 2, 3, 4, 5)
-      r1 = sc * (D(0, 0) + D(5, 1) + D(4, 2));
-      r2 = sc * (D(5, 0) + D(1, 1) + D(3, 2));
-      r3 = sc * (D(4, 0) + D(3, 1) + D(2, 2));
-      }
-      const long long v = ((long long)(z0 + p - 2) * n2 + (y0 + ty)) * n1 + (x0 + tx);
-      const float f1 = (float)r1, f2 = (float)r2, f3 = (float)r3;
-      rout[v] = f1;
-      rout[N + v] = f2;
-      rout[2 * N + v] = f3;
-      rr += f1 * f1 + f2 * f2 + f3 * f3;
-    }
-    __syncthreads();
   }
-  // per-CTA sums, fixed order
-  double q[7] = {(double)rr, ss[0], ss[1], ss[2], ss[3], ss[4], ss[5]};
-#pragma unroll
-  for (int k = 0; k < 7; ++k)
-    for (int off = 16; off > 0; off >>= 1) q[k] += __shfl_down_sync(0xffffffffu, q[k], off);
-  if ((threadIdx.x & 31) == 0) {
-#pragma unroll
-    for (int k = 0; k < 7; ++k) red[threadIdx.x >> 5][k] = q[k];
-  }
-  __syncthreads();
-  if (threadIdx.x < 7) {
-    double s = 0.0;
-    for (int w = 0; w < NT / 32; ++w) s += red[w][threadIdx.x];
-    const long long b = ((long long)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
-    part[8 * b + threadIdx.x] = s;
-  }
-}
-
-// The averaged-forward-difference case (AHC, AFB/R) of residual64_kernel with the work shared between
-// planes.  In the 2x2 window of a thread on plane z, with g_ab = f(x + a, y + b, z):
-//   Qx f = (g10 - g00) + (g11 - g01),  Qy f = (g01 - g00) + (g11 - g10),  P f = g00 + g01 + g10 + g11,
-// and D_x f(z) = Qx f(z) + Qx f(z+1), D_y f(z) = Qy f(z) + Qy f(z+1), D_z f(z) = P f(z+1) - P f(z).  So
-// r_1(z) = M_1(z) + S_1(z+1) with S_1 = Qx s11 + Qy s12 + P s13 and M_1 = Qx s11 + Qy s12 - P s13 (and
-// likewise r_2 from s12, s22, s23 and r_3 from s13, s23, s33): each plane is visited once, and only M
-// is carried to the next plane.  Same outputs and partial sums as residual64_kernel<RS_AFD>.
-__global__ void __launch_bounds__(kResTX * kResTY) residual64_afd_kernel(const double* __restrict__ eps,
-                                                                         const double* __restrict__ lam,
-                                                                         const double* __restrict__ mu,
-                                                                         const double* __restrict__ estar, Dims d,
-                                                                         double inv_h, float* __restrict__ rout,
-                                                                         double* __restrict__ part,
-                                                                         const SolveState* gate) {
-  if (gate && gate->done) return;
-  constexpr int HX = kResTX + 1, HY = kResTY + 1, NT = kResTX * kResTY;
-  __shared__ double sg[6][HY][HX];
-  __shared__ double red[NT / 32][8];
-  const int n1 = d.n1, n2 = d.n2, n3 = d.n3;
-  const long long N = d.N;
-  const int x0 = blockIdx.x * kResTX, y0 = blockIdx.y * kResTY, z0 = blockIdx.z * kResTZ;
-  const int tx = threadIdx.x % kResTX, ty = threadIdx.x / kResTX;
-  const bool col_ok = (x0 + tx < n1) && (y0 + ty < n2);
+  const bool load = t0 < HX * HY, inner = t0 < NO;
+  const bool col_ok = inner && x0 + hx - LO < n1 && y0 + hy - LO < n2;
+  const long long off = load ? (long long)((y0 + hy - LO + n2) % n2) * n1 + (x0 + hx - LO + n1) % n1 : 0;
+  const int at = hy * HX + hx;
   const int nz = min(kResTZ, n3 - z0);
-  const double sc = 0.25 * inv_h;
-  double ss[6] = {0, 0, 0, 0, 0, 0};
+  const double sc = (S == RS_AFD ? 0.25 : (S == RS_ACD ? 0.125 : 0.5)) * inv_h;
+  const bool sc2 = (__double2hiint(sc) & 0xfffff) == 0 && __double2loint(sc) == 0;  // a power of two
+  long long ss[6] = {};
   float rr = 0.f;
-  double M1 = 0.0, M2 = 0.0, M3 = 0.0;
+  long long M[1 + LO][3] = {};
+  int hmax = 0;
+  if (t0 < 2) top[t0] = 0;
+  __syncthreads();
 #pragma unroll 1
-  for (int p = 0; p <= nz; ++p) {  // planes z0 .. z0 + nz
-    const int zw = (z0 + p) % n3;
-    for (int i = threadIdx.x; i < HX * HY; i += NT) {
-      const int hx = i % HX, hy = i / HX;
-      const int xg = (x0 + hx) % n1, yg = (y0 + hy) % n2;
-      const long long v = ((long long)zw * n2 + yg) * n1 + xg;
-      double e[6];
+  for (int p = -LO; p <= nz; ++p) {  // planes z0 - LO .. z0 + nz
+    const int zw = (z0 + p + n3) % n3;
+    const long long v = (long long)zw * n1 * n2 + off;
+    double e[6], sgm[6];
 #pragma unroll
-      for (int c = 0; c < 6; ++c) e[c] = eps[c * N + v];
-      if (estar) {
+    for (int c = 0; c < 6; ++c) e[c] = eps[c * N + v];
+    const double la = lam[v], mv = mu[v];
+    if (EST) {
 #pragma unroll
-        for (int c = 0; c < 6; ++c) e[c] -= estar[c * N + v];
+      for (int c = 0; c < 6; ++c) e[c] -= estar[c * N + v];
+    }
+    const double m2 = mv + mv, ltr = la * (e[0] + e[1] + e[2]);
+    int m = 0;
+#pragma unroll
+    for (int c = 0; c < 6; ++c) {
+      sgm[c] = c < 3 ? m2 * e[c] + ltr : m2 * e[c];
+      m = max(m, fx_mag(sgm[c]));
+    }
+    if (!load) m = 0;
+    m = __reduce_max_sync(0xffffffffu, m);
+    if ((t0 & 31) == 0) atomicMax(&top[p & 1], m);
+    __syncthreads();  // also: the previous plane's window reads are over
+    const int old = hmax;
+    hmax = max(hmax, top[p & 1]);
+    const FxLine L = fx_line(hmax);
+    if (hmax > old && old > 0) {
+      const FxLine K = fx_line(old);
+      const int up = (L.e - L.off) - (K.e - K.off);
+#pragma unroll
+      for (int q = 0; q <= LO; ++q)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) asm("shr.s64 %0, %0, %1;" : "+l"(M[q][c]) : "r"(up));
+#pragma unroll
+      for (int c = 0; c < 6; ++c) asm("shr.s64 %0, %0, %1;" : "+l"(ss[c]) : "r"(up));
+    }
+    const bool own = col_ok && p >= 0 && p < nz;
+    // (far lines apart: multiplications that are predicated off still occupy the FP64 pipe)
+    if (L.far) {
+#pragma unroll 1
+      for (int c = 0; c < 6; ++c) {
+        double s = 0.0;
+#pragma unroll
+        for (int k = 0; k < 6; ++k) s = c == k ? sgm[k] : s;
+        const long long q = fx_round<58>(s * L.pin, L);
+        if (load) sg[c][at] = q;
+#pragma unroll
+        for (int k = 0; k < 6; ++k)
+          if (own && c == k) ss[k] += q;
       }
-      const double m2 = 2.0 * mu[v], ltr = lam[v] * (e[0] + e[1] + e[2]);
-      double sgm[6];
-      sgm[0] = m2 * e[0] + ltr;
-      sgm[1] = m2 * e[1] + ltr;
-      sgm[2] = m2 * e[2] + ltr;
-      sgm[3] = m2 * e[3];
-      sgm[4] = m2 * e[4];
-      sgm[5] = m2 * e[5];
+    } else {
 #pragma unroll
-      for (int c = 0; c < 6; ++c) sg[c][hy][hx] = sgm[c];
-      if (hx < kResTX && hy < kResTY && p < nz && x0 + hx < n1 && y0 + hy < n2) {
-#pragma unroll
-        for (int c = 0; c < 6; ++c) ss[c] += sgm[c];
+      for (int c = 0; c < 6; ++c) {
+        const long long q = fx_round<58>(sgm[c], L);
+        if (load) sg[c][at] = q;
+        if (own) ss[c] += q;  // at most 16 planes: 2^62
       }
     }
+    if (t0 == 0) top[(p + 1) & 1] = 0;  // (its last readers passed the barrier above)
     __syncthreads();
     if (col_ok) {
-      auto g = [&](int c, int a, int b) -> double { return sg[c][ty + b][tx + a]; };
-      // components (11, 22, 33, 23, 13, 12) = (0, 1, 2, 3, 4, 5)
-      const double qx11 = (g(0, 1, 0) - g(0, 0, 0)) + (g(0, 1, 1) - g(0, 0, 1));
-      const double qy22 = (g(1, 0, 1) - g(1, 0, 0)) + (g(1, 1, 1) - g(1, 1, 0));
-      const double p33 = (g(2, 0, 0) + g(2, 0, 1)) + (g(2, 1, 0) + g(2, 1, 1));
-      const double a12 = g(5, 1, 1) - g(5, 0, 0), b12 = g(5, 1, 0) - g(5, 0, 1);
-      const double qx12 = a12 + b12, qy12 = a12 - b12;
-      const double u13 = g(4, 1, 0) + g(4, 1, 1), w13 = g(4, 0, 0) + g(4, 0, 1);
-      const double qx13 = u13 - w13, p13 = u13 + w13;
-      const double u23 = g(3, 0, 1) + g(3, 1, 1), w23 = g(3, 0, 0) + g(3, 1, 0);
-      const double qy23 = u23 - w23, p23 = u23 + w23;
-      const double t1 = qx11 + qy12, t2 = qx12 + qy22, t3 = qx13 + qy23;
-      if (p >= 1) {  // outputs on plane z0 + p - 1
-        const double r1 = sc * (M1 + (t1 + p13));
-        const double r2 = sc * (M2 + (t2 + p23));
-        const double r3 = sc * (M3 + (t3 + p33));
-        const long long v = ((long long)(z0 + p - 1) * n2 + (y0 + ty)) * n1 + (x0 + tx);
-        const float f1 = (float)r1, f2 = (float)r2, f3 = (float)r3;
-        rout[v] = f1;
-        rout[N + v] = f2;
-        rout[2 * N + v] = f3;
-        rr += f1 * f1 + f2 * f2 + f3 * f3;
+      long long t[3], s[3];  // components (11, 22, 33, 23, 13, 12) = (0, 1, 2, 3, 4, 5)
+      if (S == RS_CD) {
+        auto dx = [&](int c) -> long long { return sg[c][at + 1] - sg[c][at - 1]; };
+        auto dy = [&](int c) -> long long { return sg[c][at + HX] - sg[c][at - HX]; };
+        t[0] = dx(0) + dy(5), t[1] = dx(5) + dy(1), t[2] = dx(4) + dy(3);
+        s[0] = sg[4][at], s[1] = sg[3][at], s[2] = sg[2][at];
+      } else {
+        constexpr int W = 1 + LO;  // the window's step
+        const int w0 = at - LO * (HX + 1);
+        auto g = [&](int c, int a, int b) -> long long { return sg[c][w0 + W * (b * HX + a)]; };
+        const long long qx11 = (g(0, 1, 0) - g(0, 0, 0)) + (g(0, 1, 1) - g(0, 0, 1));
+        const long long qy22 = (g(1, 0, 1) - g(1, 0, 0)) + (g(1, 1, 1) - g(1, 1, 0));
+        const long long p33 = (g(2, 0, 0) + g(2, 0, 1)) + (g(2, 1, 0) + g(2, 1, 1));
+        const long long a12 = g(5, 1, 1) - g(5, 0, 0), b12 = g(5, 1, 0) - g(5, 0, 1);
+        const long long u13 = g(4, 1, 0) + g(4, 1, 1), w13 = g(4, 0, 0) + g(4, 0, 1);
+        const long long u23 = g(3, 0, 1) + g(3, 1, 1), w23 = g(3, 0, 0) + g(3, 1, 0);
+        t[0] = qx11 + (a12 - b12), t[1] = (a12 + b12) + qy22, t[2] = (u13 - w13) + (u23 - w23);
+        s[0] = u13 + w13, s[1] = u23 + w23, s[2] = p33;
       }
-      M1 = t1 - p13;
-      M2 = t2 - p23;
-      M3 = t3 - p33;
+      if (p >= 1) {  // outputs on plane z0 + p - 1
+        const long long v = (long long)(z0 + p - 1) * n1 * n2 + off;
+        // value = q 2^(e - off - 1022 - 58) sc
+        const int k = L.e - L.off - 1080 + ((__double2hiint(sc) >> 20) - 1023);
+        const bool near = sc2 && k > -100 && k < 60;
+        const float f2 = __int_as_float((k + 127) << 23);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          const long long q = M[0][c] + (S == RS_CD ? s[c] : t[c] + s[c]);
+          float f;
+          if (near) f = __ll2float_rn(q) * f2;
+          else f = (float)(scalbn((double)q, L.e - L.off - 1080) * sc);
+          if (hmax >= 0x7ff00000) f = __int_as_float(0x7fc00000);
+          rout[c * N + v] = f;
+          rr += f * f;
+        }
+      }
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        if (S == RS_CD) {
+          M[0][c] = t[c] - M[LO][c];
+          M[LO][c] = s[c];
+        } else {
+          if (LO) M[0][c] = M[LO][c];
+          M[LO][c] = t[c] - s[c];
+        }
+      }
     }
-    __syncthreads();
   }
-  double q[7] = {(double)rr, ss[0], ss[1], ss[2], ss[3], ss[4], ss[5]};
+  // per-CTA sums in a fixed order; the lanes' stress sums in integers, 5 bits lower (57 bits stay)
+  const FxLine L = fx_line(hmax);
+  double r64 = rr;
 #pragma unroll
-  for (int k = 0; k < 7; ++k)
-    for (int off = 16; off > 0; off >>= 1) q[k] += __shfl_down_sync(0xffffffffu, q[k], off);
-  if ((threadIdx.x & 31) == 0) {
+  for (int off5 = 16; off5 > 0; off5 >>= 1) r64 += __shfl_down_sync(0xffffffffu, r64, off5);
 #pragma unroll
-    for (int k = 0; k < 7; ++k) red[threadIdx.x >> 5][k] = q[k];
+  for (int c = 0; c < 6; ++c) {
+    ss[c] = (ss[c] + 16) >> 5;
+#pragma unroll
+    for (int off5 = 16; off5 > 0; off5 >>= 1) ss[c] += __shfl_down_sync(0xffffffffu, ss[c], off5);
+  }
+  if (inner && (t0 & 31) == 0) {
+    red[t0 >> 5][0] = r64;
+#pragma unroll
+    for (int c = 0; c < 6; ++c)
+      red[t0 >> 5][1 + c] = hmax >= 0x7ff00000 ? __hiloint2double(0x7ff80000, 0) : scalbn((double)ss[c], L.e - L.off - 1075);
   }
   __syncthreads();
-  if (threadIdx.x < 7) {
+  if (t0 < 7) {
     double sm = 0.0;
-    for (int w = 0; w < NT / 32; ++w) sm += red[w][threadIdx.x];
+    for (int w = 0; w < NO / 32; ++w) sm += red[w][t0];
     const long long b = ((long long)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
-    part[8 * b + threadIdx.x] = sm;
+    part[8 * b + t0] = sm;
   }
 }
 
