@@ -250,9 +250,6 @@ __device__ __forceinline__ void tma_store_4d(const CUtensorMap* map, const void*
       "r"(c1), "r"(c2), "r"(c3), "r"(smem_u32(src))
       : "memory");
 }
-__device__ __forceinline__ void bulk_commit_and_wait_read() {
-  asm volatile("cp.async.bulk.commit_group;\n\tcp.async.bulk.wait_group.read 0;" ::: "memory");
-}
 
 // Byte offset inside a 512-byte-aligned region as laid out by the 64-byte TMA swizzle
 // (CU_TENSOR_MAP_SWIZZLE_64B): the 16-byte chunk index (bits 4-5) is XORed with bits 7-8.
@@ -325,7 +322,10 @@ __device__ __forceinline__ void sfft(float2* v, int t, int h, const float2* tw3,
 // [6][N rows][8 columns] of float2 in the 64-byte swizzle, so that the lane pattern of the transforms
 // (T rows of two adjacent columns per warp) and that of the Green step (4 rows x 8 columns per warp)
 // both touch each bank pair twice per warp access, the minimum for 256 bytes.  The Green step takes
-// all its FP64-residual sources from global memory in batches before its arithmetic.
+// all its FP64-residual sources from global memory in batches before its arithmetic.  Two CTAs share an SM (96 KB tiles), so a
+// CTA has to overlap its own phases too: each component has its own mbarrier and is transformed as soon as it has arrived,
+// is stored as soon as its inverse transforms are done, the source rows go to L2 meanwhile, and warps whose columns lie
+// beyond the half spectrum (seven of the last tile's eight at n1 = 256) skip the transforms: 256^3 294 -> 272 us.
 // ------------------------------------------------------------------------------------------------
 template <int N> struct SPlanOk {
   static constexpr bool ok = CPlan<N>::ok && CPlan<N>::NST == 2 && CPlan<N>::R(0) == CPlan<N>::T &&
@@ -333,6 +333,13 @@ template <int N> struct SPlanOk {
 };
 template <int N> constexpr size_t zs_smem_bytes() {
   return (size_t)6 * N * 64 + 1024 + (size_t)3 * N * sizeof(float2);
+}
+
+// The source rows of a tile (3 components x N rows x 64 bytes, used by the Green step) on their way into L2 while the tile loads.
+template <int N, int NT>
+__device__ __forceinline__ void prefetch_source(const float2* vsrc, const Dims& d, int k2, int k10) {
+  for (int i = threadIdx.x; i < 3 * N; i += NT)
+    asm volatile("prefetch.global.L2 [%0];" ::"l"(vsrc + (i / N) * d.S + d.row(i % N, k2) * d.P + k10));
 }
 
 template <int N>
@@ -351,19 +358,21 @@ __global__ void __launch_bounds__(24 * CPlan<N>::T, 2) pass_z_s_kernel(const __g
   float2* twl = reinterpret_cast<float2*>(tile + 6 * N * 64);
   float2* ab3 = twl + N;
   float2* roots = ab3 + N;
-  __shared__ __align__(8) unsigned long long bar;
+  __shared__ __align__(8) unsigned long long bar[6];
   __shared__ double red[32];
   __shared__ int abort_flag;
   const int k10 = blockIdx.x * COLS, k2 = blockIdx.y;
   if (threadIdx.x == 0) {
-    mbar_init(&bar, 1);
+    for (int c = 0; c < 6; ++c) mbar_init(&bar[c], 1);
     mbar_fence_init();
     abort_flag = 0;
   }
   __syncthreads();
   if (threadIdx.x == 0) {
-    mbar_expect_tx(&bar, 6u * N * 64u);
-    for (int c = 0; c < 6; ++c) tma_load_4d(tile + c * N * 64, &tmap, &bar, 2 * k10, k2, 0, c);
+    for (int c = 0; c < 6; ++c) {
+      mbar_expect_tx(&bar[c], N * 64u);
+      tma_load_4d(tile + c * N * 64, &tmap, &bar[c], 2 * k10, k2, 0, c);
+    }
   }
   for (int i = threadIdx.x; i < N; i += NT) {
     const int tt = i % T_, jj = i / T_;
@@ -374,20 +383,14 @@ __global__ void __launch_bounds__(24 * CPlan<N>::T, 2) pass_z_s_kernel(const __g
     ab.y = gp.B[2][i];
     ab3[i] = ab;
   }
-  if (threadIdx.x == 0 && !mbar_wait_bounded(&bar, 0)) abort_flag = 1;
+  prefetch_source<N, NT>(vsrc, d, k2, k10);
   __syncthreads();
-  if (abort_flag) {
-    if (threadIdx.x == 0) {
-      atomicExch(&st->done, (int)DONE_TIMEOUT);
-      mbar_wait_bounded(&bar, 0);  // the loads land in this CTA's shared memory: wait (bounded) for them
-    }
-    return;
-  }
   // lines interleaved in the warp: lane = LPW t + h, line = LPW warp + h
   constexpr int LPW = 32 / T_;
   const int lane = threadIdx.x & 31, h = lane % LPW, t = lane / LPW;
   const int line = (threadIdx.x >> 5) * LPW + h;
   const int col = line % COLS, compA = line / COLS;
+  const bool some = k10 + (line - h) % COLS < d.n1h;  // the warp has a column of the half spectrum
   auto el = [&](int c, int z, int cc) -> float2& {
     return *reinterpret_cast<float2*>(tile + swz64((unsigned)(c * N * 64 + z * 64 + cc * 8)));
   };
@@ -395,6 +398,8 @@ __global__ void __launch_bounds__(24 * CPlan<N>::T, 2) pass_z_s_kernel(const __g
 #pragma unroll 1
   for (int ab = 0; ab < 2; ++ab) {
     const int c = compA + 3 * ab;
+    if (!__all_sync(0xffffffffu, mbar_wait_bounded(&bar[c], 0))) { abort_flag = 1; break; }
+    if (!some) continue;
     float2 v[T_];
 #pragma unroll
     for (int r = 0; r < T_; ++r) v[r] = el(c, t + T_ * r, col);
@@ -403,6 +408,13 @@ __global__ void __launch_bounds__(24 * CPlan<N>::T, 2) pass_z_s_kernel(const __g
     for (int k = 0; k < T_; ++k) el(c, t + T_ * k, col) = v[k];
   }
   __syncthreads();
+  if (abort_flag) {
+    if (threadIdx.x == 0) {
+      atomicExch(&st->done, (int)DONE_TIMEOUT);
+      for (int c = 0; c < 6; ++c) mbar_wait_bounded(&bar[c], 0);  // the loads land in this CTA's shared memory
+    }
+    return;
+  }
   // Green step: point p = threadIdx.x + NT q is (row p / 8, column p % 8)
   float acc = 0.f;
   {
@@ -469,24 +481,26 @@ __global__ void __launch_bounds__(24 * CPlan<N>::T, 2) pass_z_s_kernel(const __g
     for (int off = 16; off > 0; off >>= 1) sm += __shfl_down_sync(0xffffffffu, sm, off);
     if (threadIdx.x == 0) partials[blockIdx.y * gridDim.x + blockIdx.x] = sm;
   }
-  // inverse transforms, in place
+  // inverse transforms, in place; a component is stored as soon as its 8 T threads are done
 #pragma unroll 1
   for (int ab = 0; ab < 2; ++ab) {
     const int c = compA + 3 * ab;
-    float2 v[T_];
+    if (some) {
+      float2 v[T_];
 #pragma unroll
-    for (int r = 0; r < T_; ++r) v[r] = el(c, t + T_ * r, col);
-    sfft<N, true, false, true>(v, t, h, twl, roots);   // phased input, true output
+      for (int r = 0; r < T_; ++r) v[r] = el(c, t + T_ * r, col);
+      sfft<N, true, false, true>(v, t, h, twl, roots);   // phased input, true output
 #pragma unroll
-    for (int k = 0; k < T_; ++k) el(c, t + T_ * k, col) = v[k];
+      for (int k = 0; k < T_; ++k) el(c, t + T_ * k, col) = v[k];
+    }
+    fence_proxy_async();  // this thread's writes before the TMA unit's reads
+    asm volatile("bar.sync %0, %1;" ::"r"(1 + compA), "n"(COLS * T_) : "memory");
+    if (threadIdx.x % (COLS * T_) == 0) {
+      tma_store_4d(&tmap, tile + c * N * 64, 2 * k10, k2, 0, c);
+      asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+    }
   }
-  // the tile back to global memory: make the generic-proxy writes visible to the TMA unit first
-  fence_proxy_async();
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int c = 0; c < 6; ++c) tma_store_4d(&tmap, tile + c * N * 64, 2 * k10, k2, 0, c);
-    bulk_commit_and_wait_read();
-  }
+  if (threadIdx.x % (COLS * T_) == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -496,7 +510,7 @@ __global__ void __launch_bounds__(24 * CPlan<N>::T, 2) pass_z_s_kernel(const __g
 // are done.  A warp transforms two neighbouring columns of one component at a time (components 0-2, then 3-5): lane t
 // holds rows t + 32 r of both, read and written as 16-byte pairs, and the stages (16, 16, 2) exchange in place in the
 // line's own rows without a CTA barrier.  The exchange permutes rows by exchange_row so that eight lanes sixteen rows apart
-// still meet eight different 16-byte slots of the 64-byte swizzle.  512^3: 4.63 ms (4 columns, ordinary loads, 32-byte rows) -> 3.00 ms, 2.7 TB/s of necessary traffic;
+// still meet eight different 16-byte slots of the 64-byte swizzle.  512^3: 4.63 ms (4 columns, ordinary loads, 32-byte rows) -> 2.96 ms, 2.7 TB/s of necessary traffic;
 // what is left is the tile that nothing overlaps: load, Green step and store of one CTA per SM follow one another.
 // ------------------------------------------------------------------------------------------------
 struct ZL {
@@ -579,8 +593,10 @@ static __global__ void __launch_bounds__(ZL::NT, 1) pass_z_l_kernel(const __grid
     twl[i] = tw[i];
     ab3[i] = make_float2(gp.A[2][i], gp.B[2][i]);
   }
+  prefetch_source<N, NT>(vsrc, d, k2, k10);
   __syncthreads();
   const int t = threadIdx.x & 31, warp = threadIdx.x >> 5, m = warp & 3;  // columns 2 m, 2 m + 1
+  const bool some = k10 + 2 * m < d.n1h;
   auto rows = [&](int c) {
     return [=](int e) { return reinterpret_cast<float4*>(tile + swz64((unsigned)((c * N + e) * 64 + m * 16))); };
   };
@@ -588,7 +604,8 @@ static __global__ void __launch_bounds__(ZL::NT, 1) pass_z_l_kernel(const __grid
 #pragma unroll 1
   for (int half = 0; half < 2; ++half) {
     const int c = (warp >> 2) + 3 * half;
-    if (!mbar_wait_bounded(&bar[c], 0)) { abort_flag = 1; break; }
+    if (!__all_sync(0xffffffffu, mbar_wait_bounded(&bar[c], 0))) { abort_flag = 1; break; }
+    if (!some) continue;
     const auto row = rows(c);
 #pragma unroll
     for (int r = 0; r < 16; ++r) {
@@ -667,20 +684,22 @@ static __global__ void __launch_bounds__(ZL::NT, 1) pass_z_l_kernel(const __grid
 #pragma unroll 1
   for (int half = 0; half < 2; ++half) {
     const int c = (warp >> 2) + 3 * half;
-    const auto row = rows(c);
+    if (some) {
+      const auto row = rows(c);
 #pragma unroll
-    for (int r = 0; r < 16; ++r) {
-      const float4 x = *row(t + 32 * r);
-      v[0][r] = make_float2(x.x, x.y);
-      v[1][r] = make_float2(x.z, x.w);
+      for (int r = 0; r < 16; ++r) {
+        const float4 x = *row(t + 32 * r);
+        v[0][r] = make_float2(x.x, x.y);
+        v[1][r] = make_float2(x.z, x.w);
+      }
+      __syncwarp();
+      zl_fft<true>(v, t, twl, row);
+#pragma unroll
+      for (int b = 0; b < 8; ++b)
+#pragma unroll
+        for (int r = 0; r < 2; ++r)
+          *row(t + 32 * b + 256 * r) = make_float4(v[0][2 * b + r].x, v[0][2 * b + r].y, v[1][2 * b + r].x, v[1][2 * b + r].y);
     }
-    __syncwarp();
-    zl_fft<true>(v, t, twl, row);
-#pragma unroll
-    for (int b = 0; b < 8; ++b)
-#pragma unroll
-      for (int r = 0; r < 2; ++r)
-        *row(t + 32 * b + 256 * r) = make_float4(v[0][2 * b + r].x, v[0][2 * b + r].y, v[1][2 * b + r].x, v[1][2 * b + r].y);
     fence_proxy_async();  // this thread's writes before the TMA unit's reads
     asm volatile("bar.sync %0, 128;" ::"r"(1 + (warp >> 2)) : "memory");  // the component's four warps
     if ((threadIdx.x & 127) == 0) {
