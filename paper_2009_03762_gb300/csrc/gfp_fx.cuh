@@ -295,6 +295,14 @@ __device__ __forceinline__ void fx_tile_line(double2* w, SL sl, int t, int line,
   fx_out<P::E>(v, w, fx_bias<60>(L, fx_shift<N>(), 0), L);
 }
 
+__device__ __forceinline__ void fx_prefetch(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
+// a / 2 without the FP64 pipe; below 2^-1021 zero
+__device__ __forceinline__ double fx_half(double a) {
+  const int hi = __double2hiint(a), e = hi & 0x7ff00000;
+  if (e == 0x7ff00000) return a;
+  return e > 0x00100000 ? __hiloint2double(hi - 0x00100000, __double2loint(a)) : 0.0;
+}
+
 // ------------------------------------------------------------------------------------------------
 // pass_y: CTA = `cols` k1 columns x all n2 rows of one component at fixed k3; thread = (column, t).
 // ------------------------------------------------------------------------------------------------
@@ -342,7 +350,9 @@ __global__ void __launch_bounds__(COLS > 0 ? COLS * FxPlan<N>::T : 1024) pass_y_
 // the first stage is register b R0 + r with j = b + r E/R0, of the last stage's output b RL + r with
 // j = b + r E/RL.  The half spectrum's two halves meet through shuffles: N - k of thread t's
 // k = t + T j is element E - 1 - j of thread T - t (of t = 0: its own element E - j).  Both transforms run through one
-// copy of the code (the inverse on swapped real and imaginary parts): two copies overflow the instruction cache.
+// copy of the code (the inverse on swapped real and imaginary parts): two copies overflow the instruction cache.  What the
+// update reads is prefetched into L2 during the inverse transform, and factors of two stay off the FP64 pipe (half of its
+// time is busy): 256^3 1.53 -> 1.50 ms, 128^3 195 -> 186 us, 64^3 31.9 -> 30.0 us.
 // ------------------------------------------------------------------------------------------------
 template <int N> __host__ __device__ constexpr int fx_line_pitch() { return N + N / 16; }
 
@@ -379,6 +389,12 @@ __global__ void __launch_bounds__(192, FxPlan<N>::E <= 8 ? 3 : 2) pass_x_fx_kern
   const long long v0 = (live ? li : 0) * N + t;
   double* ep = eps + (2 * p) * d.N + v0;
   const double E0 = p == 0 ? pp.E[0] : (p == 1 ? pp.E[2] : pp.E[4]), E1 = p == 0 ? pp.E[1] : (p == 1 ? pp.E[3] : pp.E[5]);
+  if (have_delta && live) {  // what the update reads after the inverse transform, on its way into L2
+    if (!zero)
+      for (int i = t; i < N / 8; i += T_) fx_prefetch(eps + (2 * p + (i & 1)) * d.N + li * N + (i >> 1) * 16);
+    if (p < 2)
+      for (int i = t; i < N / 16; i += T_) fx_prefetch((p ? mu : lam) + li * N + i * 16);
+  }
   __syncthreads();
   double2 w[E];  // elements x = t + T j: increment, strain, stress; around the spectrum: A and B at k = t + T j, j < E/2
 #pragma unroll 1
@@ -414,10 +430,13 @@ __global__ void __launch_bounds__(192, FxPlan<N>::E <= 8 ? 3 : 2) pass_x_fx_kern
           for (int j = 0; j < E; ++j)
             if (live) { w[j].x -= es[T_ * j]; w[j].y -= es[d.N + T_ * j]; }
         }
-        // half the stress, mu e + lambda (tr e / 2): the factor 2 goes into the exponent of the transform's results
-        if (in && p < 2) {
+        // half the stress, mu e + (lambda / 2) tr e: the factor 2 goes into the exponent of the transform's results
+        if (in && p == 0) {
 #pragma unroll
-          for (int j = 0; j < E; ++j) (p == 0 ? tr0 : tr1)[t + T_ * j] = 0.5 * (p == 0 ? w[j].x + w[j].y : w[j].x);
+          for (int j = 0; j < E; ++j) tr0[t + T_ * j] = w[j].x + w[j].y;
+        } else if (in && p == 1) {
+#pragma unroll
+          for (int j = 0; j < E; ++j) tr1[t + T_ * j] = w[j].x;
         }
         double la[E], m[E];
 #pragma unroll
@@ -429,6 +448,8 @@ __global__ void __launch_bounds__(192, FxPlan<N>::E <= 8 ? 3 : 2) pass_x_fx_kern
 #pragma unroll
           for (int j = 0; j < E; ++j) { m[j] -= pp.mu_h; la[j] -= pp.lam_h; }
         }
+#pragma unroll
+        for (int j = 0; j < E; ++j) la[j] = fx_half(la[j]);
         __syncthreads();
         if (p == 2) {
 #pragma unroll
@@ -450,11 +471,19 @@ __global__ void __launch_bounds__(192, FxPlan<N>::E <= 8 ? 3 : 2) pass_x_fx_kern
     for (int o = 1; o < T_; o <<= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
     const FxLine L = fx_line(mx);
     fx2 q[E], v[E];
-    fx_in<59, E>(w, q, L);
+    if (L.far) {  // (one branch for the elements and the one at N/2)
+#pragma unroll
+      for (int i = 0; i < E; ++i) { w[i].x *= L.pin; w[i].y *= L.pin; }
+      ny.x *= L.pin;
+      ny.y *= L.pin;
+    }
+#pragma unroll
+    for (int i = 0; i < E; ++i) { q[i].x = fx_from<59>(w[i].x, L); q[i].y = fx_from<59>(w[i].y, L); }
     if (inv) {
       // the pair's half spectra as one Hermitian-extended line: A + iB at k, conj(A) + i conj(B) at N - k
       fx2 zc[EH], nq;
-      fx_in<59, 1>(&ny, &nq, L);
+      nq.x = fx_from<59>(ny.x, L);
+      nq.y = fx_from<59>(ny.y, L);
 #pragma unroll
       for (int j = 0; j < EH; ++j) {
         const fx2 a = q[j], b = q[EH + j];
@@ -503,9 +532,16 @@ __global__ void __launch_bounds__(192, FxPlan<N>::E <= 8 ? 3 : 2) pass_x_fx_kern
         q[j].x = fx_add(z.x, zn[j].x); q[j].y = fx_sub(z.y, zn[j].y);
         q[EH + j].x = fx_add(z.y, zn[j].y); q[EH + j].y = fx_sub(zn[j].x, z.x);
       }
-      if (t == 0) fx_out<1>(&nq, &ny, bias, L);
+      if (t == 0) ny = make_double2(fx_to(nq.x, bias), fx_to(nq.y, bias));
     }
-    fx_out<E>(q, w, bias, L);
+#pragma unroll
+    for (int i = 0; i < E; ++i) w[i] = make_double2(fx_to(q[i].x, bias), fx_to(q[i].y, bias));
+    if (L.far) {
+#pragma unroll
+      for (int i = 0; i < E; ++i) { w[i].x *= L.pout; w[i].y *= L.pout; }
+      ny.x *= L.pout;
+      ny.y *= L.pout;
+    }
     if (inv) {
       if (outmode) {
 #pragma unroll
