@@ -167,7 +167,7 @@ __global__ void __launch_bounds__(512) pass_y_c_kernel(typename C<R>::T* __restr
 
 // ------------------------------------------------------------------------------------------------
 // pass_z_gamma: CTA = C columns x 6 components x all n3 rows at fixed k2; line = (comp, col).
-// Same modes as the generic kernel (PZ_GAMMA, PZ_RESIDUAL, PZ_INNER).
+// The inner iterations of the mixed solve, as the generic kernel.
 // ------------------------------------------------------------------------------------------------
 // FP32 register FFTs of up to 16 elements per thread fit two 384-thread CTAs per SM.
 template <typename R, int N> struct ZBound {
@@ -178,25 +178,21 @@ template <typename R, int N> struct ZBound {
 
 // Green step on a z-tile in shared memory: rows [k3][ZS] holding 6 components x cols columns
 // (component c, column cc at c cols + cc, XOR swz on odd rows).  Residual partial of the thread
-// (returned), T(0), and, by mode, the increment written back in place (PZ_GAMMA, PZ_INNER, PZ_DGO) or
-// the inner-iteration source stored (PZ_RESIDUAL).  vs: the tile's inner source staged as
+// (returned), the increment written back in place.  vs: the tile's inner source staged as
 // [3][N][cols], or null to read it from global memory.  blockDim.x is a multiple of cols: every
 // thread keeps one column.
 template <typename R, int N>
 __device__ __forceinline__ R green_tile(typename C<R>::T* __restrict__ buf, int ZS, int cols, int swz,
                                         const typename C<R>::T* __restrict__ ab3, const float2* vs, const Dims& d,
-                                        int k10, int k2, const GammaParams<R>& gp, SolveState* __restrict__ st,
-                                        int mode, float2* __restrict__ vsrc, R* acc2 = nullptr) {
+                                        int k10, int k2, const GammaParams<R>& gp, const float2* __restrict__ vsrc) {
   typedef typename C<R>::T T;
   R acc = 0;
-  const bool ny2 = ((d.n2 & 1) == 0) && (2 * k2 == d.n2);
   const R b2 = gp.B[1][k2], a2 = gp.A[1][k2];
   const int cc = threadIdx.x % cols;
   const int k1 = k10 + cc;
   if (k1 < d.n1h) {
     const R a1 = gp.A[0][k1], b1 = gp.B[0][k1];
-    const bool ny1 = ((d.n1 & 1) == 0) && (2 * k1 == d.n1);
-    const bool self1 = (k1 == 0) || ny1;
+    const bool self1 = (k1 == 0) || (((d.n1 & 1) == 0) && (2 * k1 == d.n1));
     const int zstep = blockDim.x / cols;
     // inner source of point z: staged tile or global memory
     auto source = [&](int z, float2& s1, float2& s2, float2& s3) {
@@ -209,13 +205,10 @@ __device__ __forceinline__ R green_tile(typename C<R>::T* __restrict__ buf, int 
     // the next point's source is loaded one point ahead, so its latency overlaps this point's arithmetic
     float2 p1, p2, p3;
     const int z0 = threadIdx.x / cols;
-    if (mode == PZ_INNER && z0 < N) source(z0, p1, p2, p3);
+    if (z0 < N) source(z0, p1, p2, p3);
     for (int z = z0; z < N; z += zstep) {
-      float2 s1, s2, s3;
-      if (mode == PZ_INNER) {
-        s1 = p1; s2 = p2; s3 = p3;
-        if (z + zstep < N) source(z + zstep, p1, p2, p3);
-      }
+      const float2 s1 = p1, s2 = p2, s3 = p3;
+      if (z + zstep < N) source(z + zstep, p1, p2, p3);
       T* rowz = buf + z * ZS;
       const int sw = (z & 1) ? swz : 0;
       T tt[6];
@@ -224,55 +217,13 @@ __device__ __forceinline__ R green_tile(typename C<R>::T* __restrict__ buf, int 
       const T ab = ab3[z];
       const R a3 = ab.x, b3 = ab.y;
       const R kt1 = a1 * b2 * b3, kt2 = a2 * b3 * b1, kt3 = a3 * b1 * b2;
-      const bool ny3 = (2 * z == N);
-      const long long vi = d.row(z, k2) * d.P + k1;
-      if (sizeof(R) == 8 && mode == PZ_DISP) {  // FP64 only (folded out of the FP32 kernels' registers)
-        T o[6];
-        disp_point<R>(tt, kt1, kt2, kt3, gp.half_shift, d, k1, k2, z, gp.invN, o);
-#pragma unroll
-        for (int c = 0; c < 6; ++c) rowz[(c * cols + cc) ^ sw] = o[c];
-        continue;
-      }
-      if (mode != PZ_INNER && k1 == 0 && k2 == 0 && z == 0) {
-#pragma unroll
-        for (int c = 0; c < 6; ++c) st->T0[c] = (double)tt[c].x;
-      }
       T v1, v2, v3;
       tk_vec<R>(tt, kt1, kt2, kt3, v1, v2, v3);
-      if (mode == PZ_INNER) {
-        v1.x += (R)s1.x; v1.y += (R)s1.y; v2.x += (R)s2.x; v2.y += (R)s2.y; v3.x += (R)s3.x; v3.y += (R)s3.y;
-      }
-      R r2 = vnorm2(v1, v2, v3);
-      if (!self1) {
-        if (gp.nyq_avg && (ny2 || ny3)) r2 += tk_norm2<R>(tt, kt1, ny2 ? -kt2 : kt2, ny3 ? -kt3 : kt3);
-        else r2 *= (R)2;
-      }
-      acc += r2;
-      if (sizeof(R) == 8 && mode == PZ_GAMMA && acc2 && gp.vprev) {  // FP64 only (the paper's stop rule)
-        const R c = incr_point<R>(v1, v2, v3, kt1, kt2, kt3, gp, vi, d.S);
-        *acc2 += self1 ? c : (R)2 * c;
-      }
-      if (mode == PZ_RESIDUAL) {
-        float2 o1, o2, o3;
-        o1.x = (float)v1.x; o1.y = (float)v1.y; o2.x = (float)v2.x; o2.y = (float)v2.y;
-        o3.x = (float)v3.x; o3.y = (float)v3.y;
-        vsrc[vi] = o1; vsrc[d.S + vi] = o2; vsrc[2 * d.S + vi] = o3;
-        continue;
-      }
+      v1.x += (R)s1.x; v1.y += (R)s1.y; v2.x += (R)s2.x; v2.y += (R)s2.y; v3.x += (R)s3.x; v3.y += (R)s3.y;
+      const R r2 = vnorm2(v1, v2, v3);
+      acc += self1 ? r2 : (R)2 * r2;
       T o[6];
-      if (mode == PZ_DGO) {
-        dgo_apply_point<R>(tt, gp.dgo, vi, d.S, gp.invN, o);
-#pragma unroll
-        for (int c = 0; c < 6; ++c) rowz[(c * cols + cc) ^ sw] = o[c];
-        continue;
-      }
       gamma0_from_v<R>(v1, v2, v3, kt1, kt2, kt3, gp.c_mu, gp.c_lm, gp.invN, o);
-      if (gp.nyq_avg && (ny1 || ny2 || ny3)) {
-        T o2[6];
-        gamma0_apply<R>(tt, ny1 ? -kt1 : kt1, ny2 ? -kt2 : kt2, ny3 ? -kt3 : kt3, gp.c_mu, gp.c_lm, gp.invN, o2);
-#pragma unroll
-        for (int c = 0; c < 6; ++c) { o[c].x = (R)0.5 * (o[c].x + o2[c].x); o[c].y = (R)0.5 * (o[c].y + o2[c].y); }
-      }
 #pragma unroll
       for (int c = 0; c < 6; ++c) rowz[(c * cols + cc) ^ sw] = o[c];
     }
@@ -285,7 +236,7 @@ template <typename R, int N, int COLS>
 __global__ void __launch_bounds__(ZBound<R, N>::threads, ZBound<R, N>::blocks) pass_z_c_kernel(typename C<R>::T* __restrict__ spec,
                                                        const typename C<R>::T* __restrict__ tw, Dims d, int cols_arg,
                                                        GammaParams<R> gp, double* __restrict__ partials,
-                                                       SolveState* __restrict__ st, int mode, float2* __restrict__ vsrc) {
+                                                       SolveState* __restrict__ st, const float2* __restrict__ vsrc) {
   typedef typename C<R>::T T;
   typedef CPlan<N> P;
   const int cols = COLS > 0 ? COLS : cols_arg;
@@ -319,7 +270,7 @@ __global__ void __launch_bounds__(ZBound<R, N>::threads, ZBound<R, N>::blocks) p
   // granule lies wholly inside or wholly beyond the row; granules at or beyond P are not copied (an
   // 8-column tile can reach past P, and past the end of the buffer on its last row), and the
   // columns they would hold are never read.)
-  const bool stage_v = (mode == PZ_INNER) && (cols == 2 || cols == 4 || cols == 8);
+  const bool stage_v = cols == 2 || cols == 4 || cols == 8;
   if (stage_v) {
     const int per_row = cols / 2;  // 16-byte granules per row
     for (int i = threadIdx.x; i < 3 * N * per_row; i += blockDim.x) {
@@ -348,15 +299,8 @@ __global__ void __launch_bounds__(ZBound<R, N>::threads, ZBound<R, N>::blocks) p
     for (int r = 0; r < RL; ++r) sl[cout_idx<N, P::NST - 1>(t, b, r)] = v[b * RL + r];
   if (stage_v) cp_async_wait_all();
   __syncthreads();
-  // Green operator, residual and T(0) per (k3, column)
-  R acc2 = 0;
-  const R acc = green_tile<R, N>(buf, ZS, cols, 0, ab3, stage_v ? vs : nullptr, d, k10, k2, gp, st, mode, vsrc,
-                                 &acc2);
-  if (sizeof(R) == 8 && mode == PZ_GAMMA && gp.vprev) {
-    const double s2 = block_sum((double)acc2, red);
-    if (threadIdx.x == 0) gp.cpart[blockIdx.y * gridDim.x + blockIdx.x] = s2;
-    __syncthreads();
-  }
+  // Green operator and residual per (k3, column)
+  const R acc = green_tile<R, N>(buf, ZS, cols, 0, ab3, stage_v ? vs : nullptr, d, k10, k2, gp, vsrc);
   double accd = (double)acc;
   for (int off = 16; off > 0; off >>= 1) accd += __shfl_down_sync(0xffffffffu, accd, off);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = accd;
@@ -367,7 +311,6 @@ __global__ void __launch_bounds__(ZBound<R, N>::threads, ZBound<R, N>::blocks) p
     for (int off = 16; off > 0; off >>= 1) s += __shfl_down_sync(0xffffffffu, s, off);
     if (threadIdx.x == 0) partials[blockIdx.y * gridDim.x + blockIdx.x] = s;
   }
-  if (mode == PZ_RESIDUAL) return;
 #pragma unroll
   for (int b = 0; b < P::E / P::R(0); ++b)
 #pragma unroll
@@ -394,7 +337,7 @@ template <typename R, int N>
 __global__ void __launch_bounds__(24 * CPlan<N>::T, 2) pass_z_c2_kernel(typename C<R>::T* __restrict__ spec,
                                                        const typename C<R>::T* __restrict__ tw, Dims d,
                                                        GammaParams<R> gp, double* __restrict__ partials,
-                                                       SolveState* __restrict__ st, int mode, float2* __restrict__ vsrc) {
+                                                       SolveState* __restrict__ st, const float2* __restrict__ vsrc) {
   typedef typename C<R>::T T;
   typedef CPlan<N> P;
   constexpr int COLS = 8, ZS = 6 * COLS;
@@ -465,7 +408,7 @@ __global__ void __launch_bounds__(24 * CPlan<N>::T, 2) pass_z_c2_kernel(typename
 #pragma unroll
     for (int r = 0; r < RL; ++r) slB[cout_idx<N, P::NST - 1>(t, b, r)] = v[b * RL + r];
   __syncthreads();
-  const R acc = green_tile<R, N>(buf, ZS, COLS, 8, ab3, nullptr, d, k10, k2, gp, st, mode, vsrc);
+  const R acc = green_tile<R, N>(buf, ZS, COLS, 8, ab3, nullptr, d, k10, k2, gp, vsrc);
   double accd = (double)acc;
   for (int off = 16; off > 0; off >>= 1) accd += __shfl_down_sync(0xffffffffu, accd, off);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = accd;
@@ -476,7 +419,6 @@ __global__ void __launch_bounds__(24 * CPlan<N>::T, 2) pass_z_c2_kernel(typename
     for (int off = 16; off > 0; off >>= 1) s += __shfl_down_sync(0xffffffffu, s, off);
     if (threadIdx.x == 0) partials[blockIdx.y * gridDim.x + blockIdx.x] = s;
   }
-  if (mode == PZ_RESIDUAL) return;
   // inverse transforms: tile -> registers -> global, line A then line B
 #pragma unroll
   for (int b = 0; b < P::E / P::R(0); ++b)
@@ -512,13 +454,11 @@ template <typename R, int N>
 __global__ void __launch_bounds__(512) pass_x_c_kernel(typename C<R>::T* __restrict__ spec, R* __restrict__ eps,
                                                        const R* __restrict__ lam, const R* __restrict__ mu,
                                                        const typename C<R>::T* __restrict__ tw, Dims d, int lines,
-                                                       int flags, PolarParams pp,
-                                                       const SolveState* __restrict__ st) {
+                                                       int flags, const SolveState* __restrict__ st) {
   typedef typename C<R>::T T;
   typedef CPlan<N> P;
   if (st->done) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ double red[32];
   T* twl = reinterpret_cast<T*>(smem_raw);
   T* buf = twl + N;                          // [3 lines][N + N/16] (padded line-major)
   constexpr int LP = N + N / 16;
@@ -532,11 +472,6 @@ __global__ void __launch_bounds__(512) pass_x_c_kernel(typename C<R>::T* __restr
   const bool live = (fl < 3 * lines) && (li < nlines);
   const bool zero = (flags & PX_ZERO) != 0 || st->restart;
   const bool have_delta = (flags & PX_DELTA) != 0 && !st->restart;
-  // eigenstrain and displacement output are FP64 features: compiled out of the FP32 instance, whose
-  // registers (64) set its occupancy
-  constexpr bool F64 = sizeof(R) == 8;
-  const bool outmode = F64 && (flags & PX_OUTPUT) != 0, strainmode = F64 && (flags & PX_STRAIN) != 0;
-  const bool dres = F64 && (flags & PX_DRES) != 0;
   const SLine<T, true> sl{buf + fl * LP, 1};
   T v[P::E];
   if (have_delta) {
@@ -566,12 +501,10 @@ __global__ void __launch_bounds__(512) pass_x_c_kernel(typename C<R>::T* __restr
       for (int r = 0; r < RL; ++r) sl[cout_idx<N, P::NST - 1>(t, b, r)] = v[b * RL + r];
   }
   __syncthreads();
-  const bool polar = (flags & PX_POLAR) != 0;
-  double dacc = 0.0;
   // XU voxels per step, all their loads issued before any store: a plain loop waits one DRAM latency
   // per voxel, since its strain loads are ordered after the previous voxel's stores to the same array
-  // (FP32: 2 voxels at 64 registers; FP64 keeps 1, its registers are already at the launch bound)
-  constexpr int XU = sizeof(R) == 4 ? 2 : 1;
+  // (2 voxels at 64 registers)
+  constexpr int XU = 2;
   const int nvox = lines * N;
   for (int i0 = threadIdx.x; i0 < nvox; i0 += XU * blockDim.x) {
     R eu[XU][6], lu[XU], mu_[XU];
@@ -582,7 +515,7 @@ __global__ void __launch_bounds__(512) pass_x_c_kernel(typename C<R>::T* __restr
       const bool ok = i < nvox && lj < nlines;
       const long long vv = lj * N + i % N;
 #pragma unroll
-      for (int c = 0; c < 6; ++c) eu[u][c] = (ok && !zero && !outmode) ? eps[c * d.N + vv] : (R)0;
+      for (int c = 0; c < 6; ++c) eu[u][c] = (ok && !zero) ? eps[c * d.N + vv] : (R)0;
       lu[u] = ok ? lam[vv] : (R)0;
       mu_[u] = ok ? mu[vv] : (R)0;
     }
@@ -605,42 +538,18 @@ __global__ void __launch_bounds__(512) pass_x_c_kernel(typename C<R>::T* __restr
         dd[2 * q] = z.x;
         dd[2 * q + 1] = z.y;
       }
-      if (outmode) {
 #pragma unroll
-        for (int c = 0; c < 3; ++c) eps[c * d.N + vv] = dd[c];
-        continue;
-      }
-      if (polar) dacc += polar_update<R>(e, dd, pp);
-      else {
-        if (dres) dacc += incr_norm2<R>(dd);
-#pragma unroll
-        for (int c = 0; c < 6; ++c) e[c] += dd[c];
-      }
+      for (int c = 0; c < 6; ++c) e[c] += dd[c];
     }
     if (have_delta || zero) {
 #pragma unroll
       for (int c = 0; c < 6; ++c) eps[c * d.N + vv] = e[c];
     }
     T zz[3];
-    if (strainmode) {
-      zz[0].x = e[0] - (R)pp.E[0]; zz[0].y = e[1] - (R)pp.E[1];
-      zz[1].x = e[2] - (R)pp.E[2]; zz[1].y = e[3] - (R)pp.E[3];
-      zz[2].x = e[4] - (R)pp.E[4]; zz[2].y = e[5] - (R)pp.E[5];
-    } else if (polar) pack_stress<R>(e, lu[u] - (R)pp.lam_h, mu_[u] - (R)pp.mu_h, zz);
-    else if (F64 && pp.estar) {
-      R es[6];
-#pragma unroll
-      for (int c = 0; c < 6; ++c) es[c] = e[c] - (R)pp.estar[c * d.N + vv];
-      pack_stress<R>(es, lu[u], mu_[u], zz);
-    } else pack_stress<R>(e, lu[u], mu_[u], zz);
+    pack_stress<R>(e, lu[u], mu_[u], zz);
 #pragma unroll
     for (int q = 0; q < 3; ++q) buf[(q * lines + ll) * LP + px] = zz[q];
     }
-  }
-  if (outmode) return;
-  if ((polar || dres) && have_delta) {
-    const double sum = block_sum(dacc, red);
-    if (threadIdx.x == 0) pp.partials[blockIdx.x] = sum;
   }
   __syncthreads();
 #pragma unroll

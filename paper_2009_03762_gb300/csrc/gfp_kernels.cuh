@@ -279,11 +279,10 @@ __device__ __forceinline__ double block_sum(double v, double* red) {
 template <typename R>
 __global__ void pass_x_kernel(typename C<R>::T* __restrict__ spec, R* __restrict__ eps, const R* __restrict__ lam,
                               const R* __restrict__ mu, const typename C<R>::T* __restrict__ tw, FftPlan plan, Dims d,
-                              int lines, int flags, PolarParams pp, const SolveState* __restrict__ st) {
+                              int lines, int flags, const SolveState* __restrict__ st) {
   typedef typename C<R>::T T;
   if (st->done) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ double red[32];
   T* twl = reinterpret_cast<T*>(smem_raw);
   T* bufa = twl + d.n1;                      // [3 pairs][lines][n1], two ping-pong copies
   T* bufb = bufa + 3 * lines * d.n1;
@@ -294,7 +293,6 @@ __global__ void pass_x_kernel(typename C<R>::T* __restrict__ spec, R* __restrict
   const long long line0 = (long long)blockIdx.x * lines;
   const bool zero = (flags & PX_ZERO) != 0 || st->restart;
   const bool have_delta = (flags & PX_DELTA) != 0 && !st->restart;
-  const bool outmode = (flags & PX_OUTPUT) != 0, strainmode = (flags & PX_STRAIN) != 0;
   for (int i = threadIdx.x; i < n1; i += blockDim.x) twl[i] = tw[i];
   const int tot_lines = 3 * lines;
   if (have_delta) {
@@ -324,9 +322,6 @@ __global__ void pass_x_kernel(typename C<R>::T* __restrict__ spec, R* __restrict
   } else {
     __syncthreads();
   }
-  const bool polar = (flags & PX_POLAR) != 0;
-  const bool dres = sizeof(R) == 8 && (flags & PX_DRES) != 0;
-  double dacc = 0.0;
   // state update, sigma = C : eps, repack sigma pairs for the forward transform
   for (int i = threadIdx.x; i < lines * n1; i += blockDim.x) {
     const int l = by_n.div(i), x = i - l * n1;
@@ -334,7 +329,7 @@ __global__ void pass_x_kernel(typename C<R>::T* __restrict__ spec, R* __restrict
     if (li >= nlines) continue;
     const long long v = li * n1 + x;
     R e[6];
-    if (zero || outmode) {
+    if (zero) {
 #pragma unroll
       for (int c = 0; c < 6; ++c) e[c] = (R)0;
     } else {
@@ -349,41 +344,17 @@ __global__ void pass_x_kernel(typename C<R>::T* __restrict__ spec, R* __restrict
         dd[2 * p] = z.x;
         dd[2 * p + 1] = z.y;
       }
-      if (outmode) {
 #pragma unroll
-        for (int c = 0; c < 3; ++c) eps[c * d.N + v] = dd[c];
-        continue;
-      }
-      if (polar) dacc += polar_update<R>(e, dd, pp);
-      else {
-        if (dres) dacc += incr_norm2<R>(dd);
-#pragma unroll
-        for (int c = 0; c < 6; ++c) e[c] += dd[c];
-      }
+      for (int c = 0; c < 6; ++c) e[c] += dd[c];
     }
     if (have_delta || zero) {
 #pragma unroll
       for (int c = 0; c < 6; ++c) eps[c * d.N + v] = e[c];
     }
     T zz[3];
-    if (strainmode) {
-      zz[0].x = e[0] - (R)pp.E[0]; zz[0].y = e[1] - (R)pp.E[1];
-      zz[1].x = e[2] - (R)pp.E[2]; zz[1].y = e[3] - (R)pp.E[3];
-      zz[2].x = e[4] - (R)pp.E[4]; zz[2].y = e[5] - (R)pp.E[5];
-    } else if (polar) pack_stress<R>(e, lam[v] - (R)pp.lam_h, mu[v] - (R)pp.mu_h, zz);
-    else if (pp.estar) {
-      R es[6];
-#pragma unroll
-      for (int c = 0; c < 6; ++c) es[c] = e[c] - (R)pp.estar[c * d.N + v];
-      pack_stress<R>(es, lam[v], mu[v], zz);
-    } else pack_stress<R>(e, lam[v], mu[v], zz);
+    pack_stress<R>(e, lam[v], mu[v], zz);
 #pragma unroll
     for (int p = 0; p < 3; ++p) buf[(p * lines + l) * n1 + x] = zz[p];
-  }
-  if (outmode) return;
-  if ((polar || dres) && have_delta) {
-    const double sum = block_sum(dacc, red);
-    if (threadIdx.x == 0) pp.partials[blockIdx.x] = sum;
   }
   __syncthreads();
   buf = fft_lines<false>(buf, buf == bufa ? bufb : bufa, twl, plan, LineLayout{tot_lines, 1, n1, false});
@@ -442,7 +413,9 @@ __global__ void pass_y_kernel(typename C<R>::T* __restrict__ spec, const typenam
 // pass_z_gamma: tile = all n3 rows x `cols` k1 columns x 6 components at fixed k2.
 // smem layout [k3][comp][col] so that line (comp, col) has element stride 6 cols.
 // --------------------------------------------------------------------------------------------
-enum { PZ_GAMMA = 0, PZ_RESIDUAL = 1, PZ_INNER = 2, PZ_DGO = 3, PZ_DISP = 4 };
+// PZ_GAMMA: Delta E = -Gamma0(kt) T / N, residual, T(0), inverse z (the FP64 iteration); PZ_INNER: the same from
+// v = T kt + vsrc (the inner iteration of the mixed solve); PZ_DGO: the tabulated discrete Green operator; PZ_DISP: below.
+enum { PZ_GAMMA = 0, PZ_INNER = 2, PZ_DGO = 3, PZ_DISP = 4 };
 
 // mode PZ_DISP (displacement output, FP64): the tile holds the transformed strain fluctuation
 // E~(k) = sym(u^(k) (x) q^a(k)) of a solution; it is replaced by u^(k) / N in components 0-2 (3-5 zeroed).
@@ -487,14 +460,13 @@ __device__ __forceinline__ void disp_point(const T t[6], R k1, R k2, R k3, int h
   }
 }
 
-// mode PZ_GAMMA: Delta E = -Gamma0(kt) T / N, residual, T(0), inverse z (the FP64 or FP32 iteration).
-// mode PZ_RESIDUAL: residual and T(0) only; stores v = T kt (FP32, [3][k3][k2][P]) as the source of
-// the inner iterations; no Green step, no inverse, the spectrum is not written back.
-// mode PZ_INNER: v = T kt + vsrc (the FP64 outer residual), residual of v, Delta E from v, inverse z.
+// Inner iterations of the mixed solve (PZ_INNER): v = T kt + vsrc (the FP64 outer residual), residual of v, Delta E = -Gamma0
+// from v, inverse z.  (The FP64 passes, in their modes, are in gfp_fx.cuh; operators that average over Nyquist partners have no mixed
+// solve.)
 template <typename R>
 __global__ void pass_z_gamma_kernel(typename C<R>::T* __restrict__ spec, const typename C<R>::T* __restrict__ tw,
                                     FftPlan plan, Dims d, int cols, GammaParams<R> gp, double* __restrict__ partials,
-                                    SolveState* __restrict__ st, int mode, float2* __restrict__ vsrc) {
+                                    SolveState* __restrict__ st, const float2* __restrict__ vsrc) {
   typedef typename C<R>::T T;
   if (st->done) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -516,9 +488,8 @@ __global__ void pass_z_gamma_kernel(typename C<R>::T* __restrict__ spec, const t
   __syncthreads();
   buf = fft_lines<false>(buf, buf2, twl, plan, LineLayout{w6, w6, 1, true});
   T* other = (buf == buf2) ? buf2 - d.n3 * w6 : buf2;
-  // Green operator, residual and T(0)
-  R acc = 0, acc2 = 0;
-  const bool ny2 = ((d.n2 & 1) == 0) && (2 * k2 == d.n2);
+  // Green operator and residual
+  R acc = 0;
   const R b2 = gp.B[1][k2], a2 = gp.A[1][k2];
   for (int i = threadIdx.x; i < d.n3 * cols; i += blockDim.x) {
     const int z = by_cols.div(i), cc = i - z * cols;
@@ -530,67 +501,18 @@ __global__ void pass_z_gamma_kernel(typename C<R>::T* __restrict__ spec, const t
     const R a1 = gp.A[0][k1], b1 = gp.B[0][k1];
     const R a3 = gp.A[2][z], b3 = gp.B[2][z];
     const R kt1 = a1 * b2 * b3, kt2 = a2 * b3 * b1, kt3 = a3 * b1 * b2;
-    const bool ny1 = ((d.n1 & 1) == 0) && (2 * k1 == d.n1);
-    const bool ny3 = ((d.n3 & 1) == 0) && (2 * z == d.n3);
-    const bool self1 = (k1 == 0) || ny1;
+    const bool self1 = (k1 == 0) || (((d.n1 & 1) == 0) && (2 * k1 == d.n1));
     const long long vi = d.row(z, k2) * d.P + k1;
-    if (mode == PZ_DISP) {
-      T o[6];
-      disp_point<R>(t, kt1, kt2, kt3, gp.half_shift, d, k1, k2, z, gp.invN, o);
-#pragma unroll
-      for (int c = 0; c < 6; ++c) buf[(z * 6 + c) * cols + cc] = o[c];
-      continue;
-    }
-    if (mode != PZ_INNER && k1 == 0 && k2 == 0 && z == 0) {
-#pragma unroll
-      for (int c = 0; c < 6; ++c) st->T0[c] = (double)t[c].x;
-    }
     T v1, v2, v3;
     tk_vec<R>(t, kt1, kt2, kt3, v1, v2, v3);
-    if (mode == PZ_INNER) {
-      const float2 s1 = vsrc[vi], s2 = vsrc[d.S + vi], s3 = vsrc[2 * d.S + vi];
-      v1.x += (R)s1.x; v1.y += (R)s1.y; v2.x += (R)s2.x; v2.y += (R)s2.y; v3.x += (R)s3.x; v3.y += (R)s3.y;
-    }
-    // residual: stored point plus (for interior k1) its Hermitian partner, whose wave vector is
-    // -kt with the components on Nyquist axes 2, 3 negated back
-    R r2 = vnorm2(v1, v2, v3);
-    if (!self1) {
-      if (gp.nyq_avg && (ny2 || ny3)) r2 += tk_norm2<R>(t, kt1, ny2 ? -kt2 : kt2, ny3 ? -kt3 : kt3);
-      else r2 *= (R)2;
-    }
-    acc += r2;
-    if (sizeof(R) == 8 && mode == PZ_GAMMA && gp.vprev) {
-      const R c = incr_point<R>(v1, v2, v3, kt1, kt2, kt3, gp, vi, d.S);
-      acc2 += self1 ? c : (R)2 * c;
-    }
-    if (mode == PZ_RESIDUAL) {
-      float2 o1, o2, o3;
-      o1.x = (float)v1.x; o1.y = (float)v1.y; o2.x = (float)v2.x; o2.y = (float)v2.y;
-      o3.x = (float)v3.x; o3.y = (float)v3.y;
-      vsrc[vi] = o1; vsrc[d.S + vi] = o2; vsrc[2 * d.S + vi] = o3;
-      continue;
-    }
+    const float2 s1 = vsrc[vi], s2 = vsrc[d.S + vi], s3 = vsrc[2 * d.S + vi];
+    v1.x += (R)s1.x; v1.y += (R)s1.y; v2.x += (R)s2.x; v2.y += (R)s2.y; v3.x += (R)s3.x; v3.y += (R)s3.y;
+    const R r2 = vnorm2(v1, v2, v3);  // the stored point plus (for interior k1) its Hermitian partner
+    acc += self1 ? r2 : (R)2 * r2;
     T o[6];
-    if (mode == PZ_DGO) {
-      dgo_apply_point<R>(t, gp.dgo, vi, d.S, gp.invN, o);
-#pragma unroll
-      for (int c = 0; c < 6; ++c) buf[(z * 6 + c) * cols + cc] = o[c];
-      continue;
-    }
     gamma0_from_v<R>(v1, v2, v3, kt1, kt2, kt3, gp.c_mu, gp.c_lm, gp.invN, o);
-    if (gp.nyq_avg && (ny1 || ny2 || ny3)) {
-      T o2[6];
-      gamma0_apply<R>(t, ny1 ? -kt1 : kt1, ny2 ? -kt2 : kt2, ny3 ? -kt3 : kt3, gp.c_mu, gp.c_lm, gp.invN, o2);
-#pragma unroll
-      for (int c = 0; c < 6; ++c) { o[c].x = (R)0.5 * (o[c].x + o2[c].x); o[c].y = (R)0.5 * (o[c].y + o2[c].y); }
-    }
 #pragma unroll
     for (int c = 0; c < 6; ++c) buf[(z * 6 + c) * cols + cc] = o[c];
-  }
-  if (sizeof(R) == 8 && mode == PZ_GAMMA && gp.vprev) {
-    const double s2 = block_sum((double)acc2, red);
-    if (threadIdx.x == 0) gp.cpart[blockIdx.y * gridDim.x + blockIdx.x] = s2;
-    __syncthreads();
   }
   // deterministic block reduction of the residual partial (FP64 across threads)
   double accd = (double)acc;
@@ -603,7 +525,6 @@ __global__ void pass_z_gamma_kernel(typename C<R>::T* __restrict__ spec, const t
     for (int off = 16; off > 0; off >>= 1) s += __shfl_down_sync(0xffffffffu, s, off);
     if (threadIdx.x == 0) partials[blockIdx.y * gridDim.x + blockIdx.x] = s;
   }
-  if (mode == PZ_RESIDUAL) return;
   buf = fft_lines<true>(buf, other, twl, plan, LineLayout{w6, w6, 1, true});
   for (int i = threadIdx.x; i < d.n3 * w6; i += blockDim.x) {
     const int z = by_w6.div(i), line = i - z * w6, comp = by_cols.div(line), cc = line - comp * cols;

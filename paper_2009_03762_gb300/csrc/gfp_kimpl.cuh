@@ -75,9 +75,9 @@ template <typename R, int N> inline int cx_lines_max() {
 template <typename R, int N>
 inline void launch_x_c(cudaStream_t s, int want_lines, int async, typename C<R>::T* spec, R* eps, const R* lam,
                        const R* mu, const typename C<R>::T* tw, const Dims& d, int flags,
-                       const PolarParams& pp, const SolveState* st) {
+                       const SolveState* st) {
   typedef typename C<R>::T T;
-  if (async && !(flags & (PX_POLAR | PX_STRAIN | PX_OUTPUT | PX_DRES)) && !pp.estar) {
+  if (async) {
     int lines = want_lines > 0 ? want_lines : 2;
     lines = std::min(lines, 512 / (3 * CPlan<N>::T));
     while (lines > 1 && xa_smem_bytes<R, N>(lines) > 200 * 1024) --lines;
@@ -93,24 +93,16 @@ inline void launch_x_c(cudaStream_t s, int want_lines, int async, typename C<R>:
   const long long nlines = (long long)d.n2 * d.n3;
   const unsigned blocks = (unsigned)((nlines + lines - 1) / lines);
   const size_t sm = cx_smem_bytes<R, N>(lines);
-  pass_x_c_kernel<R, N><<<blocks, 3 * lines * CPlan<N>::T, sm, s>>>(spec, eps, lam, mu, tw, d, lines, flags, pp, st);
+  pass_x_c_kernel<R, N><<<blocks, 3 * lines * CPlan<N>::T, sm, s>>>(spec, eps, lam, mu, tw, d, lines, flags, st);
 }
 
 template <typename R>
 void Passes<R>::pass_x(cudaStream_t s, const LaunchCfg& lc, T* spec, R* eps, const R* lam, const R* mu, const W* tw,
                        const FftPlan& plan, const Dims& d, int flags,
-                       const SolveState* st, const PolarParams* ppp) {
-  PolarParams pp;
-  if (ppp) pp = *ppp;
-  else {
-    for (int c = 0; c < 6; ++c) pp.E[c] = 0;
-    pp.lam_h = pp.mu_h = 0;
-    pp.partials = nullptr;
-    pp.estar = nullptr;
-  }
+                       const SolveState* st, const PolarParams*) {
   switch (d.n1) {
 #define GFP_CASE(N) \
-    case N: launch_x_c<R, N>(s, lc.cx_lines, lc.x_async, spec, eps, lam, mu, tw, d, flags, pp, st); return;
+    case N: launch_x_c<R, N>(s, lc.cx_lines, lc.x_async, spec, eps, lam, mu, tw, d, flags, st); return;
     GFP_FOR_CSIZES(GFP_CASE)
 #undef GFP_CASE
     default: break;
@@ -118,7 +110,7 @@ void Passes<R>::pass_x(cudaStream_t s, const LaunchCfg& lc, T* spec, R* eps, con
   const long long nlines = (long long)d.n2 * d.n3;
   const unsigned blocks = (unsigned)((nlines + lc.x_lines - 1) / lc.x_lines);
   const size_t sm = sizeof(T) * (size_t)(d.n1 + 6 * lc.x_lines * d.n1);
-  pass_x_kernel<R><<<blocks, lc.x_threads, sm, s>>>(spec, eps, lam, mu, tw, merge_stages(plan), d, lc.x_lines, flags, pp, st);
+  pass_x_kernel<R><<<blocks, lc.x_threads, sm, s>>>(spec, eps, lam, mu, tw, merge_stages(plan), d, lc.x_lines, flags, st);
 }
 
 template <typename R>
@@ -148,7 +140,7 @@ void Passes<R>::pass_y(cudaStream_t s, const LaunchCfg& lc, bool inverse, T* spe
 
 template <typename R>
 void Passes<R>::pass_z(cudaStream_t s, const LaunchCfg& lc, T* spec, const W* tw, const FftPlan& plan, const Dims& d,
-                       const GammaParams<R>& gp, double* partials, SolveState* st, int mode, float2* vsrc) {
+                       const GammaParams<R>& gp, double* partials, SolveState* st, int, float2* vsrc) {  // PZ_INNER
   const int ntx = (d.n1h + lc.z_cols - 1) / lc.z_cols;
   dim3 grid(ntx, d.n2, 1);
   switch (d.n3) {
@@ -157,7 +149,7 @@ void Passes<R>::pass_z(cudaStream_t s, const LaunchCfg& lc, T* spec, const W* tw
       const int th = 6 * lc.z_cols * CPlan<N>::T;                                                             \
       const size_t smt = sizeof(T) * (size_t)(N + 12 * N * lc.z_cols) + 128;                                 \
       if constexpr (sizeof(R) == 4 && SPlanOk<N>::ok) {                                                       \
-        if (mode == PZ_INNER && lc.z_tma && lc.ztmap && lc.z_cols == 8 && !gp.nyq_avg) {                      \
+        if (lc.z_tma && lc.ztmap && lc.z_cols == 8) {                                                         \
           pass_z_s_kernel<N><<<grid, 24 * CPlan<N>::T, zs_smem_bytes<N>(), s>>>(                              \
               *reinterpret_cast<const CUtensorMap*>(lc.ztmap), reinterpret_cast<const float2*>(tw), d,        \
               *reinterpret_cast<const GammaParams<float>*>(&gp), partials, st, vsrc);                         \
@@ -165,35 +157,35 @@ void Passes<R>::pass_z(cudaStream_t s, const LaunchCfg& lc, T* spec, const W* tw
         }                                                                                                     \
       }                                                                                                       \
       if constexpr (sizeof(R) == 4 && N == ZL::LEN) {                                                           \
-        if (mode == PZ_INNER && lc.z_tma && lc.ztmap && lc.z_cols == ZL::COLS && !gp.nyq_avg) {               \
+        if (lc.z_tma && lc.ztmap && lc.z_cols == ZL::COLS) {                                                  \
           pass_z_l_kernel<<<grid, ZL::NT, ZL::smem, s>>>(*reinterpret_cast<const CUtensorMap*>(lc.ztmap),     \
               reinterpret_cast<const float2*>(tw), d, *reinterpret_cast<const GammaParams<float>*>(&gp), partials, st, vsrc); \
           return;                                                                                             \
         }                                                                                                     \
       }                                                                                                       \
-      if (mode != PZ_DGO && mode != PZ_DISP && lc.z_tma && lc.ztmap && (lc.z_cols * sizeof(T)) % 16 == 0 && th <= 384 &&        \
+      if (lc.z_tma && lc.ztmap && (lc.z_cols * sizeof(T)) % 16 == 0 && th <= 384 &&        \
           smt <= 220 * 1024) {                    \
         const int ntiles = ntx * d.n2;                                                                        \
         const int gsz = std::min(ntiles, tma_grid<R, N>(th, smt));                                            \
         pass_z_tma_kernel<R, N><<<gsz, th, smt, s>>>(*reinterpret_cast<const CUtensorMap*>(lc.ztmap), spec, tw, \
-                                                      d, lc.z_cols, ntx, gp, partials, st, mode, vsrc,        \
+                                                      d, lc.z_cols, ntx, gp, partials, st, vsrc,              \
                                                       g_inject_tma_timeout);                                 \
         return;                                                                                               \
       }                                                                                                       \
       const size_t smc = sizeof(T) * (size_t)(2 * N + 7 * N * lc.z_cols) +                                   \
-                         (mode == PZ_INNER && (lc.z_cols == 2 || lc.z_cols == 4 || lc.z_cols == 8)                    \
+                         (lc.z_cols == 2 || lc.z_cols == 4 || lc.z_cols == 8                                          \
                               ? sizeof(float2) * 3 * N * lc.z_cols : 0);                                      \
       if constexpr (ZBound<R, N>::small) {                                                                    \
         if (lc.z_cols == 8) {                                                                                 \
           const size_t sm2 = sizeof(T) * (size_t)(2 * N + 48 * N);                                            \
-          pass_z_c2_kernel<R, N><<<grid, 24 * CPlan<N>::T, sm2, s>>>(spec, tw, d, gp, partials, st, mode, vsrc); \
+          pass_z_c2_kernel<R, N><<<grid, 24 * CPlan<N>::T, sm2, s>>>(spec, tw, d, gp, partials, st, vsrc); \
           return;                                                                                             \
         }                                                                                                     \
       }                                                                                                       \
       if (lc.z_cols == 4)                                                                                     \
-        pass_z_c_kernel<R, N, 4><<<grid, th, smc, s>>>(spec, tw, d, 4, gp, partials, st, mode, vsrc);         \
+        pass_z_c_kernel<R, N, 4><<<grid, th, smc, s>>>(spec, tw, d, 4, gp, partials, st, vsrc);         \
       else                                                                                                    \
-        pass_z_c_kernel<R, N, 0><<<grid, th, smc, s>>>(spec, tw, d, lc.z_cols, gp, partials, st, mode, vsrc); \
+        pass_z_c_kernel<R, N, 0><<<grid, th, smc, s>>>(spec, tw, d, lc.z_cols, gp, partials, st, vsrc); \
       return;                                                                                                 \
     }
     GFP_FOR_CSIZES(GFP_CASE)
@@ -201,7 +193,7 @@ void Passes<R>::pass_z(cudaStream_t s, const LaunchCfg& lc, T* spec, const W* tw
     default: break;
   }
   const size_t sm = sizeof(T) * (size_t)(d.n3 + 12 * lc.z_cols * d.n3);
-  pass_z_gamma_kernel<R><<<grid, lc.z_threads, sm, s>>>(spec, tw, merge_stages(plan), d, lc.z_cols, gp, partials, st, mode, vsrc);
+  pass_z_gamma_kernel<R><<<grid, lc.z_threads, sm, s>>>(spec, tw, merge_stages(plan), d, lc.z_cols, gp, partials, st, vsrc);
 }
 
 }  // namespace gfp

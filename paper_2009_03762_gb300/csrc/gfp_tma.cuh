@@ -69,8 +69,8 @@ __global__ void __launch_bounds__(384, ZBound<R, N>::blocks) pass_z_tma_kernel(c
                                                             typename C<R>::T* __restrict__ spec,
                                                             const typename C<R>::T* __restrict__ tw, Dims d, int cols,
                                                             int ntx, GammaParams<R> gp, double* __restrict__ partials,
-                                                            SolveState* __restrict__ st, int mode,
-                                                            float2* __restrict__ vsrc, unsigned inject_timeout) {
+                                                            SolveState* __restrict__ st,
+                                                            const float2* __restrict__ vsrc, unsigned inject_timeout) {
   typedef typename C<R>::T T;
   typedef CPlan<N> P;
   if (st->done) return;
@@ -158,9 +158,8 @@ __global__ void __launch_bounds__(384, ZBound<R, N>::blocks) pass_z_tma_kernel(c
 #pragma unroll
       for (int r = 0; r < RL; ++r) sl[cout_idx<N, P::NST - 1>(t, bb, r)] = v[bb * RL + r];
     __syncthreads();
-    // Green operator, residual and T(0) per (k3, column)
+    // Green operator and residual per (k3, column)
     R tacc = 0;
-    const bool ny2 = ((d.n2 & 1) == 0) && (2 * k2 == d.n2);
     const R b2 = gp.B[1][k2], a2 = gp.A[1][k2];
     for (int i = threadIdx.x; i < N * cols; i += blockDim.x) {
       const int cc = i % cols, z = i / cols;
@@ -172,41 +171,16 @@ __global__ void __launch_bounds__(384, ZBound<R, N>::blocks) pass_z_tma_kernel(c
       const R a1 = gp.A[0][k1], b1 = gp.B[0][k1];
       const R a3 = gp.A[2][z], b3 = gp.B[2][z];
       const R kt1 = a1 * b2 * b3, kt2 = a2 * b3 * b1, kt3 = a3 * b1 * b2;
-      const bool ny1 = ((d.n1 & 1) == 0) && (2 * k1 == d.n1);
-      const bool ny3 = (2 * z == N);
-      const bool self1 = (k1 == 0) || ny1;
+      const bool self1 = (k1 == 0) || (((d.n1 & 1) == 0) && (2 * k1 == d.n1));
       const long long vi = d.row(z, k2) * d.P + k1;
-      if (mode != PZ_INNER && k1 == 0 && k2 == 0 && z == 0) {
-#pragma unroll
-        for (int c = 0; c < 6; ++c) st->T0[c] = (double)tt[c].x;
-      }
       T v1, v2, v3;
       tk_vec<R>(tt, kt1, kt2, kt3, v1, v2, v3);
-      if (mode == PZ_INNER) {
-        const float2 s1 = vsrc[vi], s2 = vsrc[d.S + vi], s3 = vsrc[2 * d.S + vi];
-        v1.x += (R)s1.x; v1.y += (R)s1.y; v2.x += (R)s2.x; v2.y += (R)s2.y; v3.x += (R)s3.x; v3.y += (R)s3.y;
-      }
-      R r2 = vnorm2(v1, v2, v3);
-      if (!self1) {
-        if (gp.nyq_avg && (ny2 || ny3)) r2 += tk_norm2<R>(tt, kt1, ny2 ? -kt2 : kt2, ny3 ? -kt3 : kt3);
-        else r2 *= (R)2;
-      }
-      tacc += r2;
-      if (mode == PZ_RESIDUAL) {
-        float2 o1, o2, o3;
-        o1.x = (float)v1.x; o1.y = (float)v1.y; o2.x = (float)v2.x; o2.y = (float)v2.y;
-        o3.x = (float)v3.x; o3.y = (float)v3.y;
-        vsrc[vi] = o1; vsrc[d.S + vi] = o2; vsrc[2 * d.S + vi] = o3;
-        continue;
-      }
+      const float2 s1 = vsrc[vi], s2 = vsrc[d.S + vi], s3 = vsrc[2 * d.S + vi];
+      v1.x += (R)s1.x; v1.y += (R)s1.y; v2.x += (R)s2.x; v2.y += (R)s2.y; v3.x += (R)s3.x; v3.y += (R)s3.y;
+      const R r2 = vnorm2(v1, v2, v3);
+      tacc += self1 ? r2 : (R)2 * r2;
       T o[6];
       gamma0_from_v<R>(v1, v2, v3, kt1, kt2, kt3, gp.c_mu, gp.c_lm, gp.invN, o);
-      if (gp.nyq_avg && (ny1 || ny2 || ny3)) {
-        T o2[6];
-        gamma0_apply<R>(tt, ny1 ? -kt1 : kt1, ny2 ? -kt2 : kt2, ny3 ? -kt3 : kt3, gp.c_mu, gp.c_lm, gp.invN, o2);
-#pragma unroll
-        for (int c = 0; c < 6; ++c) { o[c].x = (R)0.5 * (o[c].x + o2[c].x); o[c].y = (R)0.5 * (o[c].y + o2[c].y); }
-      }
 #pragma unroll
       for (int c = 0; c < 6; ++c) buf[(c * N + z) * cols + cc] = o[c];
     }
@@ -221,21 +195,19 @@ __global__ void __launch_bounds__(384, ZBound<R, N>::blocks) pass_z_tma_kernel(c
       for (int off = 16; off > 0; off >>= 1) s += __shfl_down_sync(0xffffffffu, s, off);
       if (threadIdx.x == 0) partials[tile] = s;
     }
-    if (mode != PZ_RESIDUAL) {
 #pragma unroll
-      for (int bb = 0; bb < P::E / P::R(0); ++bb)
+    for (int bb = 0; bb < P::E / P::R(0); ++bb)
 #pragma unroll
-        for (int r = 0; r < P::R(0); ++r) v[bb * P::R(0) + r] = sl[cin_idx<N, 0>(t, bb, r)];
-      __syncthreads();
-      cfft<N, true>(v, sl, t, twl);
-      if (live) {
-        T* g = spec + comp * d.S + d.row(0, k2) * d.P + k10 + col;
-        const long long zs = d.zstride();
+      for (int r = 0; r < P::R(0); ++r) v[bb * P::R(0) + r] = sl[cin_idx<N, 0>(t, bb, r)];
+    __syncthreads();
+    cfft<N, true>(v, sl, t, twl);
+    if (live) {
+      T* g = spec + comp * d.S + d.row(0, k2) * d.P + k10 + col;
+      const long long zs = d.zstride();
 #pragma unroll
-        for (int bb = 0; bb < P::E / RL; ++bb)
+      for (int bb = 0; bb < P::E / RL; ++bb)
 #pragma unroll
-          for (int r = 0; r < RL; ++r) g[cout_idx<N, P::NST - 1>(t, bb, r) * zs] = v[bb * RL + r];
-      }
+        for (int r = 0; r < RL; ++r) g[cout_idx<N, P::NST - 1>(t, bb, r) * zs] = v[bb * RL + r];
     }
     fence_proxy_async();  // order this tile's generic shared accesses before the next async load into it
     __syncthreads();      // both the tile buffer and red[] are free for the next tile
@@ -421,8 +393,6 @@ __global__ void __launch_bounds__(24 * CPlan<N>::T, 2) pass_z_s_kernel(const __g
     const int cc = threadIdx.x & 7;
     const int k1 = k10 + cc;
     const bool live = k1 < d.n1h;
-    const bool ny2 = ((d.n2 & 1) == 0) && (2 * k2 == d.n2);
-    (void)ny2;
     const float b2 = gp.B[1][k2], a2 = gp.A[1][k2];
     const float a1 = live ? gp.A[0][k1] : 0.f, b1 = live ? gp.B[0][k1] : 0.f;
     const bool self1 = (k1 == 0) || (((d.n1 & 1) == 0) && (2 * k1 == d.n1));
