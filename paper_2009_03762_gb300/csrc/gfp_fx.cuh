@@ -8,9 +8,10 @@
 // integer instructions.  A line's error is at most a few 2^-60 of its largest element per stage, where
 // FP64 butterflies lose 2^-53 of the intermediate values.
 //
-// Measured at 256^3 (FP64 butterflies -> fixed point): x-pass 4.65 -> 1.53 ms, y-pass 1.90 -> 0.58 ms, z-pass
-// 5.34 -> 1.91 ms; the strain's error against torch's FP64 transforms after three iterations 2.27e-16 -> 1.93e-16.  The
-// passes are now bound by instruction issue (about 2.5 of 4 per clock), half of it the conversions.
+// Measured at 256^3 (FP64 butterflies -> fixed point): x-pass 4.65 -> 1.48 ms, y-pass 1.90 -> 0.50 ms, z-pass
+// 5.34 -> 1.82 ms; the strain's error against torch's FP64 transforms after three iterations 2.27e-16 -> 1.93e-16.  The
+// passes are now bound by latency at 18 to 24 warps per SM (about 2 instructions of 4 issued per clock), half of the instructions
+// being the conversions.
 //
 // Ranges: |re|, |im| < 2^60 at the input of a line, so that moduli stay below 2^60.5; a radix-4 layer grows
 // them to 2^62.5 < 2^63, and each following layer first scales by 1/4 -- for free where the element takes a
@@ -352,12 +353,13 @@ __global__ void __launch_bounds__(COLS > 0 ? COLS * FxPlan<N>::T : 1024) pass_y_
 // k = t + T j is element E - 1 - j of thread T - t (of t = 0: its own element E - j).  Both transforms run through one
 // copy of the code (the inverse on swapped real and imaginary parts): two copies overflow the instruction cache.  What the
 // update reads is prefetched into L2 during the inverse transform, and factors of two stay off the FP64 pipe (half of its
-// time is busy): 256^3 1.53 -> 1.50 ms, 128^3 195 -> 186 us, 64^3 31.9 -> 30.0 us.
+// time is busy): 256^3 1.53 -> 1.50 ms, 128^3 195 -> 186 us, 64^3 31.9 -> 30.0 us.  Four CTAs per SM at 80 registers, with up to
+// 180 bytes of spills, against three at 96: 1.48 ms, 178 us, 25.5 us.
 // ------------------------------------------------------------------------------------------------
 template <int N> __host__ __device__ constexpr int fx_line_pitch() { return N + N / 16; }
 
 template <int N>
-__global__ void __launch_bounds__(192, FxPlan<N>::E <= 8 ? 3 : 2) pass_x_fx_kernel(double2* __restrict__ spec, double* __restrict__ eps,
+__global__ void __launch_bounds__(192, FxPlan<N>::E <= 8 ? 4 : 2) pass_x_fx_kernel(double2* __restrict__ spec, double* __restrict__ eps,
                                                         const double* __restrict__ lam, const double* __restrict__ mu,
                                                         const fxw* __restrict__ tw, Dims d, int lines, int flags,
                                                         PolarParams pp, const SolveState* __restrict__ st) {
