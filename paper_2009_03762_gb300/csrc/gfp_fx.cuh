@@ -392,7 +392,7 @@ __global__ void __launch_bounds__(192, FxPlan<N>::E <= 8 ? 4 : 2) pass_x_fx_kern
   double* ep = eps + (2 * p) * d.N + v0;
   const double E0 = p == 0 ? pp.E[0] : (p == 1 ? pp.E[2] : pp.E[4]), E1 = p == 0 ? pp.E[1] : (p == 1 ? pp.E[3] : pp.E[5]);
   if (have_delta && live) {  // what the update reads after the inverse transform, on its way into L2
-    if (!zero)
+    if (!zero && !outmode)  // (the output mode's eps holds three components)
       for (int i = t; i < N / 8; i += T_) fx_prefetch(eps + (2 * p + (i & 1)) * d.N + li * N + (i >> 1) * 16);
     if (p < 2)
       for (int i = t; i < N / 16; i += T_) fx_prefetch((p ? mu : lam) + li * N + i * 16);
