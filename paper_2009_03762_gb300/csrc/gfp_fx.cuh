@@ -741,6 +741,8 @@ __device__ __forceinline__ long long fx_dot3(fxs a, fxs b, fxs c, const fxs n[3]
 __device__ __forceinline__ int fx_absh(long long q) { const int h = (int)(q >> 32); return h ^ (h >> 31); }
 __device__ __forceinline__ long long fx_sar(long long q, int d) { asm("shr.s64 %0, %0, %1;" : "+l"(q) : "r"(d)); return q; }
 __device__ __forceinline__ long long fx_shl(long long q, int d) { return (long long)((unsigned long long)q << d); }
+// The shift that fills the word: |re|, |im| <= 2^(63 - result); 63 for zero.
+__device__ __forceinline__ int fx_lead(fx2 v) { return __clzll((v.x ^ (v.x >> 63)) | (v.y ^ (v.y >> 63))) - 1; }
 
 constexpr int kFxBad = 1 << 28;  // exponent of a line with an infinity or a NaN
 
@@ -812,10 +814,10 @@ __device__ __forceinline__ int fx_green_point(const fx2 t[6], const int U[6], co
 }
 
 // All points of a tile: get(z, c, cc) and put(z, c, cc, value) the tile's elements, unit(c, cc) a line's unit, and
-// pexp(z, cc) the place of the point's exponent; top[cc] receives the column's largest (from INT_MIN).
+// pexp(z, cc) the place of the point's exponent.
 template <typename Get, typename Put, typename Unit, typename Pexp>
 __device__ __forceinline__ void fx_green_fixed(int n3, int cols, int k10, int k2, const Dims& d, const GammaParams<double>& gp,
-                                               const FxGreen& G, SolveState* __restrict__ st, int* top, double& acc, Get get,
+                                               const FxGreen& G, SolveState* __restrict__ st, double& acc, Get get,
                                                Put put, Unit unit, Pexp pexp) {
   const int nt = (int)blockDim.x / cols * cols;  // threads beyond the last whole row sit out
   if ((int)threadIdx.x >= nt) return;
@@ -825,7 +827,7 @@ __device__ __forceinline__ void fx_green_fixed(int n3, int cols, int k10, int k2
   const double a1 = gp.A[0][k1], b1 = gp.B[0][k1], a2 = gp.A[1][k2], b2 = gp.B[1][k2];
   const double f1 = a1 * b2, f2 = a2 * b1, f3 = b1 * b2;  // kt = (f1 b3, f2 b3, f3 a3)
   const double wgt = self1 ? 1.0 : 2.0;  // the stored point and its Hermitian partner
-  int U[6], best = -(1 << 30);
+  int U[6];
 #pragma unroll
   for (int c = 0; c < 6; ++c) U[c] = unit(c, cc);
   const int half = n3 / 2;
@@ -848,17 +850,17 @@ __device__ __forceinline__ void fx_green_fixed(int n3, int cols, int k10, int k2
 #pragma unroll
         for (int c = 0; c < 6; ++c) st->T0[c] = U[c] == kFxBad ? __hiloint2double(0x7ff80000, 0) : scalbn((double)t[c].x, U[c]);
       }
-      const int P = fx_green_point(t, U, n, s, wgt, G, acc, o);
-      best = max(best, P);
-      pexp(zz, cc) = P;
+      pexp(zz, cc) = fx_green_point(t, U, n, s, wgt, G, acc, o);
 #pragma unroll
       for (int c = 0; c < 6; ++c) put(zz, c, cc, o[c]);
     }
   }
-  atomicMax(&top[cc], best);
 }
 
-// Line scale of a column for the inverse transform: elements o >> (top - P + 3) of unit 2^(top + 13 + ef).
+// Line scale for the inverse transform, each line's own (with one scale per column of six lines, components that are small
+// beside the others lost bits: 64 x 64 x 512, shear increments under an axial load, rms error 4.9e-15 of them, now 1.5e-15;
+// z-pass at 256^3 1.91 -> 1.94 ms): an element o of a point with exponent P fills the word shifted left by L = fx_lead(o) and then has the exponent P - L;
+// with top the line's largest, elements go in shifted right by top - (P - L) + 3 from there, in the unit 2^(top + 13 + ef).
 struct FxBack {
   int bias;
   bool far;
@@ -1030,15 +1032,17 @@ pass_z_fxf_kernel(double2* __restrict__ spec, const fxw* __restrict__ tw, Dims d
   fxw* twl = reinterpret_cast<fxw*>(tile + 6 * N * cols);
   int* pexp = reinterpret_cast<int*>(twl + N);
   __shared__ double red[32];
-  __shared__ int emax[2][64], top[32];
+  __shared__ int emax[2][64], top[2][64];
   const int w3 = 3 * cols;
   const int l = threadIdx.x % w3, t = threadIdx.x / w3;
   const int comp0 = l / cols, col = l % cols;
   const int k10 = blockIdx.x * cols, k2 = blockIdx.y;
   const bool live = k10 + col < d.n1h;
   for (int i = threadIdx.x; i < N; i += blockDim.x) twl[i] = tw[i];
-  for (int i = threadIdx.x; i < 2 * w3; i += blockDim.x) emax[i / w3][i % w3] = 0;
-  for (int i = threadIdx.x; i < cols; i += blockDim.x) top[i] = -(1 << 30);
+  for (int i = threadIdx.x; i < 2 * w3; i += blockDim.x) {
+    emax[i / w3][i % w3] = 0;
+    top[i / w3][i % w3] = -(1 << 30);
+  }
   const long long zs = d.zstride();
   __syncthreads();
 #pragma unroll 1
@@ -1063,19 +1067,29 @@ pass_z_fxf_kernel(double2* __restrict__ spec, const fxw* __restrict__ tw, Dims d
       const FxLine L = fx_line(emax[ph][l]);
       fx_in<60, P::E>(w, v, L);
     } else {
-      const int tc = top[col];
-      back = fx_back(tc, G.ef, fx_shift<N>());
+      int ex[P::E], mx = -(1 << 30);
 #pragma unroll
       for (int b = 0; b < P::E / R0; ++b)
 #pragma unroll
         for (int r = 0; r < R0; ++r) {
-          const int z = fin_idx<N, 0>(t, b, r);
-          const int sh = tc - pexp[z * cols + col] + 3;
+          const int i = b * R0 + r, z = fin_idx<N, 0>(t, b, r);
           const fx2 x = sl[z];
-          v[b * R0 + r].x = fx_sar(x.y, sh);  // the inverse transform is the forward one between swaps of the parts
-          v[b * R0 + r].y = fx_sar(x.x, sh);
+          const int lead = fx_lead(x);
+          ex[i] = pexp[z * cols + col] - lead;
+          mx = max(mx, ex[i]);
+          v[i].x = fx_shl(x.y, lead);  // the inverse transform is the forward one between swaps of the parts
+          v[i].y = fx_shl(x.x, lead);
         }
+      atomicMax(&top[ph - 2][l], mx);
       __syncthreads();
+      const int tc = top[ph - 2][l];
+      back = fx_back(tc, G.ef, fx_shift<N>());
+#pragma unroll
+      for (int i = 0; i < P::E; ++i) {
+        const int sh = tc - ex[i] + 3;
+        v[i].x = fx_sar(v[i].x, sh);
+        v[i].y = fx_sar(v[i].y, sh);
+      }
     }
     fx_fft<N, false, false>(v, sl, t, twl);
     if (!inv) {
@@ -1099,7 +1113,7 @@ pass_z_fxf_kernel(double2* __restrict__ spec, const fxw* __restrict__ tw, Dims d
     if (ph == 1) {
       __syncthreads();
       double acc = 0.0;
-      fx_green_fixed(N, cols, k10, k2, d, gp, G, st, top, acc,
+      fx_green_fixed(N, cols, k10, k2, d, gp, G, st, acc,
                      [&](int z, int c, int cc) { return tile[(c * N + z) * cols + cc]; },
                      [&](int z, int c, int cc, fx2 o) { tile[(c * N + z) * cols + cc] = o; },
                      [&](int c, int cc) { return fx_unit(emax[c >= 3][(c >= 3 ? c - 3 : c) * cols + cc], fx_shift<N>()); },
@@ -1370,13 +1384,15 @@ __global__ void __launch_bounds__(512) pass_z_fxg_kernel(double2* __restrict__ s
   double2* buf2 = buf + n * w6;
   int* pexp = reinterpret_cast<int*>(buf2 + n * w6);  // [n][cols], FIXED only
   __shared__ double red[32];
-  __shared__ int emax[2][384], top[64];
+  __shared__ int emax[2][384];  // largest high words of the lines; back: FIXED their exponents
   const int k10 = blockIdx.x * cols, k2 = blockIdx.y;
   const LineLayout L{w6, w6, 1, true};
   const FastDiv by_cols(cols), by_w6(w6);
   for (int i = threadIdx.x; i < n; i += blockDim.x) twl[i] = tw[i];
-  for (int i = threadIdx.x; i < w6; i += blockDim.x) emax[0][i] = emax[1][i] = 0;
-  for (int i = threadIdx.x; i < cols; i += blockDim.x) top[i] = -(1 << 30);
+  for (int i = threadIdx.x; i < w6; i += blockDim.x) {
+    emax[0][i] = 0;
+    emax[1][i] = FIXED ? -(1 << 30) : 0;
+  }
   for (int i = threadIdx.x; i < n * w6; i += blockDim.x) {
     const int z = by_w6.div(i), line = i - z * w6, comp = by_cols.div(line), k1 = k10 + line - comp * cols;
     buf[i] = k1 < d.n1h ? spec[comp * d.S + d.row(z, k2) * d.P + k1] : make_double2(0.0, 0.0);
@@ -1387,7 +1403,7 @@ __global__ void __launch_bounds__(512) pass_z_fxg_kernel(double2* __restrict__ s
   double2* tile = reinterpret_cast<double2*>(r);
   double acc = 0.0, acc2 = 0.0;
   if (FIXED) {
-    fx_green_fixed(n, cols, k10, k2, d, gp, G, st, top, acc,
+    fx_green_fixed(n, cols, k10, k2, d, gp, G, st, acc,
                    [&](int z, int c, int cc) { return r[(z * 6 + c) * cols + cc]; },
                    [&](int z, int c, int cc, fx2 o) { r[(z * 6 + c) * cols + cc] = o; },
                    [&](int c, int cc) { return fx_unit(emax[0][c * cols + cc], sh); },
@@ -1409,12 +1425,20 @@ __global__ void __launch_bounds__(512) pass_z_fxg_kernel(double2* __restrict__ s
   const double s = block_sum(acc, red);  // synchronises the CTA after the Green step's writes
   if (threadIdx.x == 0) partials[cta] = s;
   if (FIXED) {
+    const int per = max(1, (int)blockDim.x / w6);  // threads per line, as in fx_tile_in
+    for (int q = threadIdx.x; q < per * w6; q += blockDim.x) {
+      const int c = by_w6.div(q), line = q - c * w6, cc = line - by_cols.div(line) * cols;
+      int m = -(1 << 30);
+      for (int z = c; z < n; z += per) m = max(m, pexp[z * cols + cc] - fx_lead(r[z * w6 + line]));
+      atomicMax(&emax[1][line], m);
+    }
+    __syncthreads();
     for (int i = threadIdx.x; i < n * w6; i += blockDim.x) {
       const int z = by_w6.div(i), line = i - z * w6, cc = line - by_cols.div(line) * cols;
-      const int down = top[cc] - pexp[z * cols + cc] + 3;
       fx2 v = r[i];
-      v.x = fx_sar(v.x, down);
-      v.y = fx_sar(v.y, down);
+      const int lead = fx_lead(v), down = emax[1][line] - (pexp[z * cols + cc] - lead) + 3;
+      v.x = fx_sar(fx_shl(v.x, lead), down);
+      v.y = fx_sar(fx_shl(v.y, lead), down);
       r[i] = v;
     }
     __syncthreads();
@@ -1428,7 +1452,7 @@ __global__ void __launch_bounds__(512) pass_z_fxg_kernel(double2* __restrict__ s
     if (k1 >= d.n1h) continue;
     double2 w;
     if (FIXED) {
-      const FxBack B = fx_back(top[line - comp * cols], G.ef, sh);
+      const FxBack B = fx_back(emax[1][line], G.ef, sh);
       w = make_double2(fx_to(r[i].x, B.bias), fx_to(r[i].y, B.bias));
       if (B.far) { w.x *= B.pout; w.y *= B.pout; }
     } else {
