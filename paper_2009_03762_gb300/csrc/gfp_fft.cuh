@@ -190,6 +190,7 @@ struct FftPlan {
   int n;
   int nst;
   int radix[12];
+  unsigned post;  // FP64 passes (fx_plan): bits by which elements are scaled down before the next stage, 2 bits of it per stage
 };
 
 // Lines live in shared memory: element e of line l at buf[l * ls + e * es].
@@ -232,6 +233,7 @@ inline FftPlan merge_stages(const FftPlan& p) {
     m.radix[s] = prod;
   }
   for (int s = m.nst; s < 12; ++s) m.radix[s] = 0;
+  m.post = 0;
   return m;
 }
 

@@ -1,12 +1,10 @@
 // FP64 line transforms in 64-bit block fixed point (sm_103a).
 //
-// GB300 issues 2 FP64 operations per clock and SM but about 62 64-bit integer additions or 32 x 32 -> 64
-// multiply-adds (both measured), so a transform held in 64-bit integers runs its butterflies an order of
-// magnitude faster than one held in doubles, and rounds less: every line is scaled by its own largest
-// exponent and carries 60 bits of it, against the 53 bits of a double.  The fields stay doubles in memory; a
-// pass converts a line's elements on the way in (fx_from) and its results on the way out (fx_to), both with
-// integer instructions.  A line's error is at most a few 2^-60 of its largest element per stage, where
-// FP64 butterflies lose 2^-53 of the intermediate values.
+// GB300 issues 2 FP64 operations per clock and SM but about 60 64-bit integer additions or 62 32 x 32 -> 64
+// multiply-adds (measured), so a transform held in 64-bit integers runs its butterflies an order of
+// magnitude faster than one held in doubles: every line is scaled by its own largest exponent and enters with 60 bits
+// of it (59 in the x-pass).  The fields stay doubles in memory; a pass converts a line's elements on the way in (fx_from)
+// and its results on the way out (fx_to), both with integer instructions.
 //
 // Measured at 256^3 (FP64 butterflies -> fixed point): x-pass 4.65 -> 1.48 ms, y-pass 1.90 -> 0.50 ms, z-pass
 // 5.34 -> 1.82 ms; the strain's error against torch's FP64 transforms after three iterations 2.27e-16 -> 1.93e-16.  The
@@ -14,9 +12,14 @@
 // being the conversions.
 //
 // Ranges: |re|, |im| < 2^60 at the input of a line, so that moduli stay below 2^60.5; a radix-4 layer grows
-// them to 2^62.5 < 2^63, and each following layer first scales by 1/4 -- for free where the element takes a
-// twiddle (Q62 twiddles, the product's upper 64 bits), with a rounded shift otherwise.  fx_shift counts the
-// scaling, and fx_to folds it into the exponent.
+// them to 2^62.5 < 2^63, and the following layers first scale by 1/4 or 1/2 -- for free where the element takes a
+// twiddle (Q62 twiddles, the product's upper 64 bits), with a rounded shift otherwise.  fx_shift counts the scaling, and
+// fx_to folds it into the exponent.
+//
+// Precision: scaled down by S = fx_shift bits in all, a line ends in units of 2^(S - 60) of its largest element (2^(S - 59) in the
+// x-pass), S within 0.3 bits of log2 n at most: 2^-54 at 256 points, 2^-52 at 512 and 729.  A line whose transform spreads over its
+// elements grows by sqrt(n) and more and keeps more bits than a double; one that is a single element (the inverse
+// transform of one mode) does not grow, and from 512 points on rounds like a double or up to 4 times coarser.
 #pragma once
 #include "gfp_fxnum.cuh"
 #include "gfp_tma.cuh"
@@ -222,8 +225,8 @@ template <int N, int S> __device__ __forceinline__ int fout_idx(int t, int b, in
   return (j / Ns) * Ns * R + (j % Ns) + r * Ns;
 }
 
-// Bits by which the elements are scaled down before the stage that follows one of radix R, and inside
-// a stage of radix R.
+// Bits by which the elements of a register plan are scaled down before the stage that follows one of radix R (other
+// schedules: FftPlan::post), and inside a stage of radix R.
 __host__ __device__ constexpr int fx_post(int R) { return R == 8 || R == 6 || R == 2 ? 1 : 2; }
 __host__ __device__ constexpr int fx_inner(int R) { return R == 18 ? 3 : (R >= 6 ? 2 : 0); }
 template <int N> __host__ __device__ constexpr int fx_shift() {
@@ -234,8 +237,27 @@ template <int N> __host__ __device__ constexpr int fx_shift() {
 }
 inline __host__ __device__ int fx_shift(const FftPlan& p) {
   int s = 0;
-  for (int q = 0; q < p.nst; ++q) s += fx_inner(p.radix[q]) + (q + 1 < p.nst ? fx_post(p.radix[q]) : 0);
+  for (int q = 0; q < p.nst; ++q) s += fx_inner(p.radix[q]) + (int)(p.post >> (2 * q) & 3);
   return s;
+}
+// A schedule as the FP64 passes run it: merged, and scaled down before each stage by the smaller of 1 and 2 bits that keeps moduli
+// below 2^62.85 (tracked in thousandths of a bit, log2 3 = 1.585).  With fx_post everywhere 729 lost 10 bits, now 8: displacements
+// of a laminate 1.5 times as far off as in FP64, now 0.5; 864 lost 9, now 8.
+inline FftPlan fx_plan(const FftPlan& p) {
+  FftPlan m = merge_stages(p);
+  int bits = 60500;
+  for (int s = 0; s < m.nst; ++s) {
+    const int R = m.radix[s];
+    const int first = R == 2 ? 1000 : (R % 3 == 0 && R != 12 ? 1585 : 2000);  // growth by the stage's first layer
+    if (s > 0) {
+      const unsigned down = bits - 1000 + first <= 62850 ? 1 : 2;
+      m.post |= down << (2 * (s - 1));
+      bits -= 1000 * (int)down;
+    }
+    const int grow = R == 2 || R == 8 ? 1000 : (R == 3 || R == 12 ? 1585 : (R == 6 ? 585 : (R == 9 || R == 18 ? 1170 : 2000)));
+    bits += grow;  // over the stage, less its own fx_inner
+  }
+  return m;
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -1185,7 +1207,7 @@ __device__ __forceinline__ fx2* fx_lines(fx2* a, fx2* b, const fxw* tw, const Ff
       default: fx_stage_lines<16, INV>(src, dst, tw, P.n, Ns, post, L); break;
     }
     Ns *= R;
-    post = fx_post(R);
+    post = (int)(P.post >> (2 * s)) & 3;
     fx2* t = src; src = dst; dst = t;
   }
   return src;

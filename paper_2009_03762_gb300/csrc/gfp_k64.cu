@@ -133,7 +133,7 @@ void Passes<double>::pass_x(cudaStream_t s, const LaunchCfg& lc, double2* spec, 
   const long long nlines = (long long)d.n2 * d.n3;
   const unsigned blocks = (unsigned)((nlines + lc.x_lines - 1) / lc.x_lines);
   const size_t sm = 16 * (size_t)(d.n1 + 6 * lc.x_lines * d.n1);
-  pass_x_fxg_kernel<<<blocks, lc.x_threads, sm, s>>>(spec, eps, lam, mu, tw, merge_stages(plan), d, lc.x_lines, flags, pp, st);
+  pass_x_fxg_kernel<<<blocks, lc.x_threads, sm, s>>>(spec, eps, lam, mu, tw, fx_plan(plan), d, lc.x_lines, flags, pp, st);
 }
 
 template <>
@@ -151,8 +151,8 @@ void Passes<double>::pass_y(cudaStream_t s, const LaunchCfg& lc, bool inverse, d
   }
   const dim3 grid((d.n1h + lc.y_cols - 1) / lc.y_cols, d.n3, comps);
   const size_t sm = 16 * (size_t)(d.n2 + 2 * lc.y_cols * d.n2);
-  if (inverse) pass_y_fxg_kernel<true><<<grid, lc.y_threads, sm, s>>>(spec, tw, merge_stages(plan), d, lc.y_cols, st);
-  else pass_y_fxg_kernel<false><<<grid, lc.y_threads, sm, s>>>(spec, tw, merge_stages(plan), d, lc.y_cols, st);
+  if (inverse) pass_y_fxg_kernel<true><<<grid, lc.y_threads, sm, s>>>(spec, tw, fx_plan(plan), d, lc.y_cols, st);
+  else pass_y_fxg_kernel<false><<<grid, lc.y_threads, sm, s>>>(spec, tw, fx_plan(plan), d, lc.y_cols, st);
 }
 
 template <>
@@ -170,9 +170,9 @@ void Passes<double>::pass_z(cudaStream_t s, const LaunchCfg& lc, double2* spec, 
   FxGreen G;
   if (fx_green_params(gp, mode, G))
     pass_z_fxg_kernel<true><<<grid, lc.z_threads, sm + sizeof(int) * (size_t)(d.n3 * lc.z_cols), s>>>(
-        spec, tw, merge_stages(plan), d, lc.z_cols, gp, G, partials, st, mode);
+        spec, tw, fx_plan(plan), d, lc.z_cols, gp, G, partials, st, mode);
   else
-    pass_z_fxg_kernel<false><<<grid, lc.z_threads, sm, s>>>(spec, tw, merge_stages(plan), d, lc.z_cols, gp, G, partials, st, mode);
+    pass_z_fxg_kernel<false><<<grid, lc.z_threads, sm, s>>>(spec, tw, fx_plan(plan), d, lc.z_cols, gp, G, partials, st, mode);
 }
 
 template struct Passes<double>;
