@@ -681,6 +681,14 @@ std::vector<FftPlan> plan_candidates(int n) {
 
 int round32(int x) { return ((x + 31) / 32) * 32; }
 
+// Widest default z-tile: register-FFT z-pass, 6 zc (n3 / 16) threads <= 512 (FP32 at 512: 4 columns 4.63, 2 columns 7.77 ms),
+// and two tile copies within a CTA's shared memory.
+int wide_z_cols(const Dims& d, int eb) {
+  int zc = d.n3 >= 512 && (eb == 16 || d.n3 != 512) ? 2 : 4;
+  while (zc > 1 && (long long)(d.n3 + 12 * zc * d.n3) * eb > 200 * 1024) zc /= 2;
+  return std::max(1, std::min(zc, d.n1h));
+}
+
 // Tile shapes per pass, bounded by the shared memory of one CTA (two ping-pong tile copies plus
 // the twiddles) and by 32-byte row segments in the strided y/z passes.
 LaunchCfg make_cfg(const Dims& d, int eb) {
@@ -703,9 +711,7 @@ LaunchCfg make_cfg(const Dims& d, int eb) {
   while (yc > 1 && (long long)(d.n2 + 2 * yc * d.n2) * eb > budget) yc /= 2;
   c.y_cols = std::max(1, std::min(yc, d.n1h));
   c.y_threads = clampt(c.y_cols * d.n2 / 8);
-  // register-FFT z-pass: 6 zc (n3 / 16) threads <= 512 (FP32 at 512: 4 columns 4.63, 2 columns 7.77 ms)
-  int zc = d.n3 >= 512 && (eb == 16 || d.n3 != 512) ? 2 : 4;
-  while (zc > 1 && (long long)(d.n3 + 12 * zc * d.n3) * eb > budget) zc /= 2;
+  int zc = wide_z_cols(d, eb);
   // lengths without a register plan: 2 columns (FP32 162^3: 239 us, 4 columns 344; FP64 162^3 834 against 903, 54^3 37 against 61
   // us), one where those CTAs would not fill the chip twice or a column is long (FP64 243^3: 2945 against 3222 us)
   if (!has_register_plan(d.n3))
@@ -1970,7 +1976,7 @@ int gfp_solve_noalloc(int n1, int n2, int n3, double h, const double* lambda, co
   d.P = ((d.n1h + 3) / 4) * 4;
   d.N = (long long)n1 * n2 * n3;
   d.S = (long long)n3 * n2 * d.P;
-  const LaunchCfg lc = make_cfg(d, 16);
+  LaunchCfg lc = make_cfg(d, 16);
   const int ns[3] = {n1, n2, n3};
   const int sblocks = 256;  // phase statistics partials
   // scratch layout: spectrum, twiddles, tables, residual partials, state, phase statistics
@@ -1980,7 +1986,15 @@ int gfp_solve_noalloc(int n1, int n2, int n3, double h, const double* lambda, co
   for (int r = 0; r < 3; ++r) { o_tw[r] = off; off = align256(off + sizeof(fxw) * ns[r]); }
   for (int r = 0; r < 3; ++r) { o_A[r] = off; off = align256(off + sizeof(double) * ns[r]); }
   for (int r = 0; r < 3; ++r) { o_B[r] = off; off = align256(off + sizeof(double) * ns[r]); }
-  const size_t o_part = off; off = align256(off + sizeof(double) * (size_t)lc.z_blocks);
+  const size_t o_part = off;
+  // a residual partial per z-tile: a grid that fits with wide tiles only takes them (512 x 324 x 1: 41796 partials with the
+  // default two columns, 21060 with four)
+  const size_t rest = align256(sizeof(SolveState)) + align256(sizeof(double) * 4 * sblocks) + align256(sizeof(unsigned long long));
+  while (o_part + align256(sizeof(double) * (size_t)lc.z_blocks) + rest > kNoAllocScratchBytes && lc.z_cols < wide_z_cols(d, 16)) {
+    lc.z_cols = std::min(2 * lc.z_cols, wide_z_cols(d, 16));
+    finalize_cfg(d, lc);
+  }
+  off = align256(off + sizeof(double) * (size_t)lc.z_blocks);
   const size_t o_st = off; off = align256(off + sizeof(SolveState));
   const size_t o_mm = off; off = align256(off + sizeof(double) * 4 * sblocks);
   const size_t o_bad = off; off = align256(off + sizeof(unsigned long long));
