@@ -246,18 +246,17 @@ __global__ void __launch_bounds__(ResHalo<S>::NT) residual_fx_kernel(const doubl
   }
 }
 
-// Mean stress of an FP64 strain field with compensated summation: sigma = C : (eps - estar) per voxel.  A thread adds the
-// stresses of four voxels in FP64 (their rounding, 2^-53 of four terms, averages out over N / 4 groups to below 1e-18 of
-// the mean at 64^3) and gathers these sums with their rounding errors (TwoSum); pairs (sum, errors) are combined the same way
+// Mean stress of an FP64 strain field with compensated summation: sigma = C : (eps - estar) per voxel.  A thread gathers
+// its voxels' stresses with their rounding errors (TwoSum, every addition: sums of several voxels in plain FP64 would round alike
+// wherever the stress repeats, as in layers, up to 1.4 units of 2^-53 of the mean); pairs (sum, errors) are combined the same way
 // by a warp per component, per CTA into part[12 b + 2 c] and by mean_stress64_final_kernel in a fixed order.  The sum the transform
 // forms at k = 0 rounds at about 1e-16 of the mean stress, which is the size of the change one voxel's modulus makes in
-// the effective stiffness of a 128^3 cell; this sum keeps the rounding well below it.  FP64 operations bound it (31 a voxel;
-// one compensated addition per voxel took 55) with the serial ends before: 256^3 2.16 + 0.16 ->
-// 0.82 + 0.01 ms, 32^3 87 + 152 -> 13 + 5 us.
+// the effective stiffness of a 128^3 cell; this sum keeps the rounding well below it.  FP64 operations bound it (55 a voxel):
+// 256^3 1.73 ms (0.82 with groups of four in plain FP64), 32^3 23 us.
 struct SumErr {
   double s, e;
   __device__ __forceinline__ void add(double x) {
-    const double t = s + x, v = t - s;
+    const double t = __dadd_rn(s, x), v = t - s;  // (a product x is not to be fused into the sum)
     e += (s - (t - v)) + (x - v);
     s = t;
   }
@@ -283,24 +282,26 @@ __global__ void __launch_bounds__(256) mean_stress64_kernel(const double* __rest
   SumErr a[6] = {};
   const long long step = (long long)gridDim.x * blockDim.x;
   for (long long v0 = blockIdx.x * (long long)blockDim.x + threadIdx.x; v0 < N; v0 += 4 * step) {
-    double x[6] = {0, 0, 0, 0, 0, 0};
+    double e[4][6], l[4], m[4];  // four voxels' loads in flight
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       const long long v = v0 + q * step;
-      if (v >= N) continue;
-      double e[6];
+      const bool in = v < N;
+      l[q] = in ? lam[v] : 0.0;
+      m[q] = in ? mu[v] : 0.0;
 #pragma unroll
-      for (int c = 0; c < 6; ++c) e[c] = eps[c * N + v];
-      if (estar) {
+      for (int c = 0; c < 6; ++c) e[q][c] = in ? eps[c * N + v] : 0.0;
+      if (estar && in) {
 #pragma unroll
-        for (int c = 0; c < 6; ++c) e[c] -= estar[c * N + v];
+        for (int c = 0; c < 6; ++c) e[q][c] -= estar[c * N + v];
       }
-      const double m2 = 2.0 * mu[v], ltr = lam[v] * (e[0] + e[1] + e[2]);
-#pragma unroll
-      for (int c = 0; c < 6; ++c) x[c] += c < 3 ? m2 * e[c] + ltr : m2 * e[c];
     }
 #pragma unroll
-    for (int c = 0; c < 6; ++c) a[c].add(x[c]);
+    for (int q = 0; q < 4; ++q) {
+      const double m2 = 2.0 * m[q], ltr = l[q] * (e[q][0] + e[q][1] + e[q][2]);
+#pragma unroll
+      for (int c = 0; c < 6; ++c) a[c].add(c < 3 ? m2 * e[q][c] + ltr : m2 * e[q][c]);
+    }
   }
 #pragma unroll
   for (int c = 0; c < 6; ++c) sh[c][threadIdx.x] = a[c];
