@@ -152,14 +152,15 @@ void Passes<R>::pass_z(cudaStream_t s, const LaunchCfg& lc, T* spec, const W* tw
         if (lc.z_tma && lc.ztmap && lc.z_cols == 8) {                                                         \
           pass_z_s_kernel<N><<<grid, 24 * CPlan<N>::T, zs_smem_bytes<N>(), s>>>(                              \
               *reinterpret_cast<const CUtensorMap*>(lc.ztmap), reinterpret_cast<const float2*>(tw), d,        \
-              *reinterpret_cast<const GammaParams<float>*>(&gp), partials, st, vsrc);                         \
+              *reinterpret_cast<const GammaParams<float>*>(&gp), partials, st, vsrc, g_inject_tma_timeout);   \
           return;                                                                                             \
         }                                                                                                     \
       }                                                                                                       \
       if constexpr (sizeof(R) == 4 && N == ZL::LEN) {                                                           \
         if (lc.z_tma && lc.ztmap && lc.z_cols == ZL::COLS) {                                                  \
           pass_z_l_kernel<<<grid, ZL::NT, ZL::smem, s>>>(*reinterpret_cast<const CUtensorMap*>(lc.ztmap),     \
-              reinterpret_cast<const float2*>(tw), d, *reinterpret_cast<const GammaParams<float>*>(&gp), partials, st, vsrc); \
+              reinterpret_cast<const float2*>(tw), d, *reinterpret_cast<const GammaParams<float>*>(&gp), partials, st, vsrc, \
+              g_inject_tma_timeout);                                                                          \
           return;                                                                                             \
         }                                                                                                     \
       }                                                                                                       \

@@ -51,6 +51,14 @@ __device__ __forceinline__ bool mbar_wait_bounded(unsigned long long* bar, unsig
   return true;
 }
 
+// Bounded wait for the first phase of n barriers, one budget for all.
+__device__ __forceinline__ void mbar_drain(unsigned long long* bars, int n, long long budget = (1LL << 31)) {
+  const long long t0 = clock64();
+  for (int i = 0; i < n; ++i)
+    while (!mbar_try_wait(&bars[i], 0))
+      if (clock64() - t0 > budget) return;
+}
+
 __device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
 __device__ __forceinline__ void tma_load_4d(void* dst, const CUtensorMap* map, unsigned long long* bar, int c0, int c1,
@@ -320,7 +328,8 @@ __global__ void __launch_bounds__(24 * CPlan<N>::T, 2) pass_z_s_kernel(const __g
                                                                       GammaParams<float> gp,
                                                                       double* __restrict__ partials,
                                                                       SolveState* __restrict__ st,
-                                                                      const float2* __restrict__ vsrc) {
+                                                                      const float2* __restrict__ vsrc,
+                                                                      unsigned inject_timeout) {
   constexpr int T_ = CPlan<N>::T, COLS = 8, NT = 24 * T_;
   if (st->done) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -330,12 +339,12 @@ __global__ void __launch_bounds__(24 * CPlan<N>::T, 2) pass_z_s_kernel(const __g
   float2* twl = reinterpret_cast<float2*>(tile + 6 * N * 64);
   float2* ab3 = twl + N;
   float2* roots = ab3 + N;
-  __shared__ __align__(8) unsigned long long bar[6];
+  __shared__ __align__(8) unsigned long long bar[7];  // one per component; [6] is never arrived at
   __shared__ double red[32];
   __shared__ int abort_flag;
   const int k10 = blockIdx.x * COLS, k2 = blockIdx.y;
   if (threadIdx.x == 0) {
-    for (int c = 0; c < 6; ++c) mbar_init(&bar[c], 1);
+    for (int c = 0; c < 7; ++c) mbar_init(&bar[c], 1);
     mbar_fence_init();
     abort_flag = 0;
   }
@@ -370,7 +379,9 @@ __global__ void __launch_bounds__(24 * CPlan<N>::T, 2) pass_z_s_kernel(const __g
 #pragma unroll 1
   for (int ab = 0; ab < 2; ++ab) {
     const int c = compA + 3 * ab;
-    if (!__all_sync(0xffffffffu, mbar_wait_bounded(&bar[c], 0))) { abort_flag = 1; break; }
+    // inject_timeout as in pass_z_tma_kernel
+    const bool ok = mbar_wait_bounded(&bar[inject_timeout ? 6 : c], 0, inject_timeout ? 1LL << 22 : 1LL << 31);
+    if (!__all_sync(0xffffffffu, ok)) { abort_flag = 1; break; }
     if (!some) continue;
     float2 v[T_];
 #pragma unroll
@@ -383,7 +394,7 @@ __global__ void __launch_bounds__(24 * CPlan<N>::T, 2) pass_z_s_kernel(const __g
   if (abort_flag) {
     if (threadIdx.x == 0) {
       atomicExch(&st->done, (int)DONE_TIMEOUT);
-      for (int c = 0; c < 6; ++c) mbar_wait_bounded(&bar[c], 0);  // the loads land in this CTA's shared memory
+      mbar_drain(bar, 6);  // the loads land in this CTA's shared memory
     }
     return;
   }
@@ -536,19 +547,19 @@ static __global__ void __launch_bounds__(ZL::NT, 1) pass_z_l_kernel(const __grid
                                                                     const float2* __restrict__ tw, Dims d,
                                                                     GammaParams<float> gp, double* __restrict__ partials,
                                                                     SolveState* __restrict__ st,
-                                                                    const float2* __restrict__ vsrc) {
+                                                                    const float2* __restrict__ vsrc, unsigned inject_timeout) {
   constexpr int N = ZL::LEN, COLS = ZL::COLS, NT = ZL::NT;
   if (st->done) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   unsigned char* tile = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);  // as in pass_z_s_kernel
   float2* twl = reinterpret_cast<float2*>(tile + ZL::tile);
   float2* ab3 = twl + N;
-  __shared__ __align__(8) unsigned long long bar[6];
+  __shared__ __align__(8) unsigned long long bar[7];  // one per component; [6] is never arrived at
   __shared__ double red[32];
   __shared__ int abort_flag;
   const int k10 = blockIdx.x * COLS, k2 = blockIdx.y;
   if (threadIdx.x == 0) {
-    for (int c = 0; c < 6; ++c) mbar_init(&bar[c], 1);
+    for (int c = 0; c < 7; ++c) mbar_init(&bar[c], 1);
     mbar_fence_init();
     abort_flag = 0;
   }
@@ -574,7 +585,9 @@ static __global__ void __launch_bounds__(ZL::NT, 1) pass_z_l_kernel(const __grid
 #pragma unroll 1
   for (int half = 0; half < 2; ++half) {
     const int c = (warp >> 2) + 3 * half;
-    if (!__all_sync(0xffffffffu, mbar_wait_bounded(&bar[c], 0))) { abort_flag = 1; break; }
+    // inject_timeout as in pass_z_tma_kernel
+    const bool ok = mbar_wait_bounded(&bar[inject_timeout ? 6 : c], 0, inject_timeout ? 1LL << 22 : 1LL << 31);
+    if (!__all_sync(0xffffffffu, ok)) { abort_flag = 1; break; }
     if (!some) continue;
     const auto row = rows(c);
 #pragma unroll
@@ -595,7 +608,7 @@ static __global__ void __launch_bounds__(ZL::NT, 1) pass_z_l_kernel(const __grid
   if (abort_flag) {
     if (threadIdx.x == 0) {
       atomicExch(&st->done, (int)DONE_TIMEOUT);
-      for (int c = 0; c < 6; ++c) mbar_wait_bounded(&bar[c], 0);  // the loads land in this CTA's shared memory
+      mbar_drain(bar, 6);  // the loads land in this CTA's shared memory
     }
     return;
   }
