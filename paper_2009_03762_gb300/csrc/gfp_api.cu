@@ -508,10 +508,13 @@ __global__ void batch_arm_kernel(SolveState* __restrict__ st, SolveState* __rest
 
 // Last kernel of a slot's window: counts the window and sets the slot's loop condition, so that the
 // slot's while-node runs another window while its outer state is running and the window budget lasts.
-// The count rises by one per window, so every slot's loop ends after at most max_windows windows.
-__global__ void batch_loop_kernel(cudaGraphConditionalHandle h, const SolveState* __restrict__ st,
-                                  int* __restrict__ windows, const BatchCtl* __restrict__ ctl) {
+// The count rises by one per window, so every slot's loop ends after at most max_windows windows.  A wait that
+// ran out in the window's inner iterations ends the slot.
+__global__ void batch_loop_kernel(cudaGraphConditionalHandle h, SolveState* __restrict__ st,
+                                  const SolveState* __restrict__ st_in, int* __restrict__ windows,
+                                  const BatchCtl* __restrict__ ctl) {
   if (threadIdx.x != 0 || blockIdx.x != 0) return;
+  if (st->done == 0 && st_in->done == DONE_TIMEOUT) st->done = DONE_TIMEOUT;
   const int w = *windows + 1;
   *windows = w;
   cudaGraphSetConditional(h, (st->done == 0 && w < ctl->max_windows) ? 1u : 0u);
@@ -2433,7 +2436,7 @@ cudaError_t batch_build_graph(gfp_batch b) {
     if (e != cudaSuccess) break;
     const GammaParams<float> gp32 = gamma_params<float>(s.g, b->sc.op, s.g->tabA32, s.g->tabB32);
     slot_window(s, b->sc.op, gp32, b->ctl, b->windows + i, kBatchWindow);
-    batch_loop_kernel<<<1, 32, 0, s.stream>>>(h, s.st, b->windows + i, b->ctl);
+    batch_loop_kernel<<<1, 32, 0, s.stream>>>(h, s.st, s.st_in, b->windows + i, b->ctl);
     cudaGraph_t captured = nullptr;
     e = cudaStreamEndCapture(s.stream, &captured);
   }
