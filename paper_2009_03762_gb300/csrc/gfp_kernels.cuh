@@ -586,6 +586,7 @@ extern unsigned g_inject_tma_timeout;
 
 template <typename R> bool cz_cols_ok(int n3, int cols);
 template <typename R> bool cz_tma_ok(int n3, int cols);
+bool cz_swizzled(int n3, int cols);  // the FP32 z-pass of such TMA-fed tiles reads the 64-byte swizzle
 template <typename R> int cy_cols_max(int n2);
 
 }  // namespace gfp
