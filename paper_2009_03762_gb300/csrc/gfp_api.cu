@@ -15,6 +15,7 @@
 #include "../../include/gfp.h"
 #include "gfp_kernels.cuh"
 #include "gfp_outer.cuh"
+#include "gfp_zmap.h"
 
 using namespace gfp;
 
@@ -682,8 +683,6 @@ std::vector<FftPlan> plan_candidates(int n) {
   return out;
 }
 
-int round32(int x) { return ((x + 31) / 32) * 32; }
-
 // Widest default z-tile: register-FFT z-pass, 6 zc (n3 / 16) threads <= 512 (FP32 at 512: 4 columns 4.63, 2 columns 7.77 ms),
 // and two tile copies within a CTA's shared memory.
 int wide_z_cols(const Dims& d, int eb) {
@@ -770,60 +769,10 @@ fxw fx_twiddle_entry(int n, int j) {
   return w;
 }
 
-// cuTensorMapEncodeTiled from the driver (looked up once; null if unavailable).
-PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
-  static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
-  static bool tried = false;
-  if (!tried) {
-    tried = true;
-    void* p = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) == cudaSuccess &&
-        q == cudaDriverEntryPointSuccess)
-      fn = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(p);
-  }
-  return fn;
-}
-
-// Tensor map of a half spectrum (FP32 or FP64 complex) as reals {2P, n2, n3, 6} with z-tiles of
-// `cols` columns x min(n3, 256) rows.  FP32 tiles of 8 columns (64-byte rows) use the 64-byte swizzle at the lengths whose
-// z-pass reads it (pass_z_s_kernel, pass_z_l_kernel), all others none.  Returns false if the shape is not TMA-eligible.
-bool encode_ztmap(CUtensorMap* m, const void* spec, const Dims& d, int cols, int real_bytes) {
-  PFN_cuTensorMapEncodeTiled_v12000 enc = tensor_map_encoder();
-  if (!enc || cols < 1 || (2 * cols * real_bytes) % 16 != 0 || ((uintptr_t)spec & 15) != 0) return false;
-  const cuuint64_t es = (cuuint64_t)real_bytes;
-  cuuint64_t dims[4] = {(cuuint64_t)(2 * d.P), (cuuint64_t)d.n2, (cuuint64_t)d.n3, 6};
-  cuuint64_t strides[3] = {2 * (cuuint64_t)d.P * es, (cuuint64_t)d.n2 * 2 * d.P * es, (cuuint64_t)d.S * 2 * es};
-  cuuint32_t box[4] = {(cuuint32_t)(2 * cols), 1, (cuuint32_t)std::min(d.n3, 256), 1};
-  cuuint32_t estr[4] = {1, 1, 1, 1};
-  const CUresult r = enc(m, real_bytes == 4 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 4,
-                         const_cast<void*>(spec), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                         (real_bytes == 4 && cz_swizzled(d.n3, cols)) ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_NONE,
-                         CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-                         CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  return r == CUDA_SUCCESS;
-}
-
-// Recompute the thread counts and partial-sum count after a tile change.
-void finalize_cfg(const Dims& d, LaunchCfg& c) {
-  auto clampt = [](int t) { return std::min(512, std::max(64, round32(t))); };
-  c.x_threads = clampt(3 * c.x_lines * d.n1 / 8);
-  c.y_threads = clampt(c.y_cols * d.n2 / 8);
-  c.z_threads = clampt(6 * c.z_cols * d.n3 / 8);
-  c.z_blocks = ((d.n1h + c.z_cols - 1) / c.z_cols) * d.n2;
-}
-
-// (Re)encode the z-tile tensor map of a launch configuration; without TMA the pass falls back to
-// the register-FFT kernel with ordinary loads.
+// (Re)encode the z-tile tensor map of a grid's launch configuration.
 void refresh_ztmap(gfp_grid g, bool mixed) {
-  LaunchCfg& lc = mixed ? g->lc32 : g->lc64;
-  CUtensorMap* m = mixed ? &g->zmap32 : &g->zmap64;
-  lc.ztmap = encode_ztmap(m, g->spec, g->d, lc.z_cols, mixed ? 4 : 8) ? m : nullptr;
-  if (!lc.ztmap && mixed && g->d.n3 == 512 && lc.z_cols == 8) {  // only the TMA-fed kernel has this width
-    lc.z_cols = 4;
-    lc.z_tma = 0;
-    finalize_cfg(g->d, lc);
-  }
+  if (mixed) attach_ztmap(g->lc32, &g->zmap32, g->spec, g->d, true);
+  else attach_ztmap(g->lc64, &g->zmap64, g->spec, g->d, false);
 }
 
 // Per-axis tables with exact zeros (kappa from the storage index; Nyquist is kappa = -n/2)
@@ -2510,8 +2459,8 @@ int gfp_batch_create(int count, gfp_grid* grids, const gfp_scheme* sc, gfp_batch
       if (e != cudaSuccess) break;
       s.lc64 = g->lc64;
       s.lc32 = g->lc32;
-      s.lc64.ztmap = encode_ztmap(&s.zm64, s.spec, d, s.lc64.z_cols, 8) ? &s.zm64 : nullptr;
-      s.lc32.ztmap = encode_ztmap(&s.zm32, s.spec, d, s.lc32.z_cols, 4) ? &s.zm32 : nullptr;
+      attach_ztmap(s.lc64, &s.zm64, s.spec, d, false);
+      attach_ztmap(s.lc32, &s.zm32, s.spec, d, true);
     }
   A((void**)&b->ctl, sizeof(BatchCtl));
   A((void**)&b->windows, sizeof(int) * nslots);
@@ -2542,8 +2491,8 @@ int gfp_batch_solve(gfp_batch b, double tol, int maxit, double* C_eff_out, int* 
       s.lc64 = s.g->lc64;
       s.lc32 = s.g->lc32;
       const Dims& d = s.g->d;
-      s.lc64.ztmap = encode_ztmap(&s.zm64, s.spec, d, s.lc64.z_cols, 8) ? &s.zm64 : nullptr;
-      s.lc32.ztmap = encode_ztmap(&s.zm32, s.spec, d, s.lc32.z_cols, 4) ? &s.zm32 : nullptr;
+      attach_ztmap(s.lc64, &s.zm64, s.spec, d, false);
+      attach_ztmap(s.lc32, &s.zm32, s.spec, d, true);
     }
     e = batch_build_graph(b);
   }
