@@ -204,17 +204,20 @@ int gfp_time_passes(gfp_grid g, const gfp_scheme* scheme, int iters, double pass
  * as radix-16, -8 or -4 stages, the radix-3 stages first or last) and keeps the fastest
  * (gfp_get_plans reads them).  tiles_out (may be
  * NULL) receives {x lines, y columns, z columns}, the x entry negated when the x-pass stages its loads
- * with cp.async and the z entry negated when the TMA z-pass is chosen.
+ * with cp.async (mixed precision only) and the z entry negated when the TMA z-pass is chosen.
  * The strain state is modified; call before a solve. */
 int gfp_tune(gfp_grid g, const gfp_scheme* scheme, int iters, int tiles_out[3]);
 
 /* Apply tile shapes for one precision (GFP_FP64 or GFP_MIXED), e.g. read from a tuning cache, in the
- * format gfp_tune returns; invalid shapes return GFP_ERR_ARG. */
+ * format gfp_tune returns; invalid shapes return GFP_ERR_ARG.  More x lines than a CTA takes run as the most
+ * it takes (FP64: 192 threads, at three component pairs of n1 / 4 to n1 / 16 threads a line), and the FP64 x-pass ignores the sign of
+ * the x entry. */
 int gfp_set_tiles(gfp_grid g, int prec, const int tiles[3]);
 
 /* Radix schedules of the shared-memory Stockham passes for one precision (GFP_FP64 or GFP_MIXED), one per
  * axis: nst[r] stages with radices radix[12 r .. 12 r + nst[r] - 1], each in {2, 3, 4, 8, 16}, their
- * product n_r (unused entries 0).  gfp_set_plans applies schedules read back from gfp_get_plans (e.g. a
+ * product n_r (unused entries 0).  Neighbouring stages run merged where their product is 6, 9, 12, 18 or one of these,
+ * in the least number of stages, so schedules that merge alike run alike.  gfp_set_plans applies schedules read back from gfp_get_plans (e.g. a
  * tuning cache); a schedule whose product is not n_r, with another radix or more than 12 stages returns
  * GFP_ERR_ARG.  Lengths with a register-FFT plan use these schedules only in the FP32 transforms of the
  * mixed solve's FP64 residual. */

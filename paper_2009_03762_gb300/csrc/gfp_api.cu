@@ -650,13 +650,16 @@ bool plan_ok(const FftPlan& p, int n) {
 
 // Candidate radix schedules of the shared-memory Stockham passes for the autotuner: the power of two
 // split into radices 16, 8 or 4 (the remainder as one smaller stage), the radix-3 stages first or last,
-// and the default; duplicates removed.
+// and the default; those that run as the same merged stages once.
 std::vector<FftPlan> plan_candidates(int n) {
   std::vector<FftPlan> out;
   auto add = [&](const FftPlan& p) {
     if (!plan_ok(p, n)) return;
-    for (const FftPlan& q : out)
-      if (q.nst == p.nst && std::equal(q.radix, q.radix + q.nst, p.radix)) return;
+    const FftPlan m = merge_stages(p);
+    for (const FftPlan& r : out) {
+      const FftPlan q = merge_stages(r);
+      if (q.nst == m.nst && std::equal(q.radix, q.radix + q.nst, m.radix)) return;
+    }
     out.push_back(p);
   };
   add(make_plan(n));
@@ -2124,7 +2127,7 @@ int gfp_tune(gfp_grid g, const gfp_scheme* sc, int iters, int tiles_out[3]) {
     LaunchCfg best = lc;
     float bt = run(0, lc);
     for (int L : cands) {
-      for (int xa = 0; xa < 2; ++xa) {
+      for (int xa = 0; xa < (mixed ? 2 : 1); ++xa) {  // (the FP64 x-pass has no cp.async variant)
         LaunchCfg c = lc;
         c.cx_lines = L;
         c.x_async = xa;
@@ -2179,7 +2182,10 @@ int gfp_tune(gfp_grid g, const gfp_scheme* sc, int iters, int tiles_out[3]) {
       if (cands.size() < 2) continue;
       LaunchCfg best = lc;
       float bt = run(r, lc);
+      const FftPlan now = merge_stages(lc.plan[r]);
       for (const FftPlan& p : cands) {
+        const FftPlan m = merge_stages(p);
+        if (m.nst == now.nst && std::equal(m.radix, m.radix + m.nst, now.radix)) continue;
         LaunchCfg c = lc;
         c.plan[r] = p;
         const float t = run(r, c);
