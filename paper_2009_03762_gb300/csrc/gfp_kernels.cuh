@@ -171,13 +171,6 @@ __device__ __forceinline__ void gamma0_from_v(T v1, T v2, T v3, R k1, R k2, R k3
   out[5].x = -(a * (k1 * v2.x + k2 * v1.x) - k1 * k2 * bkv.x); out[5].y = -(a * (k1 * v2.y + k2 * v1.y) - k1 * k2 * bkv.y);
 }
 
-template <typename R, typename T>
-__device__ __forceinline__ void gamma0_apply(const T t[6], R k1, R k2, R k3, R c_mu, R c_lm, R scale, T out[6]) {
-  T v1, v2, v3;
-  tk_vec<R>(t, k1, k2, k3, v1, v2, v3);
-  gamma0_from_v<R>(v1, v2, v3, k1, k2, k3, c_mu, c_lm, scale, out);
-}
-
 template <typename T>
 __device__ __forceinline__ auto vnorm2(T v1, T v2, T v3) -> decltype(v1.x) {
   return v1.x * v1.x + v1.y * v1.y + v2.x * v2.x + v2.y * v2.y + v3.x * v3.x + v3.y * v3.y;
