@@ -305,7 +305,8 @@ __device__ __forceinline__ void sfft(float2* v, int t, int h, const float2* tw3,
 // all its FP64-residual sources from global memory in batches before its arithmetic.  Two CTAs share an SM (96 KB tiles), so a
 // CTA has to overlap its own phases too: each component has its own mbarrier and is transformed as soon as it has arrived,
 // is stored as soon as its inverse transforms are done, the source rows go to L2 meanwhile, and warps whose columns lie
-// beyond the half spectrum (seven of the last tile's eight at n1 = 256) skip the transforms: 256^3 294 -> 272 us.
+// beyond the half spectrum (seven of the last tile's eight at n1 = 256) skip the transforms: 256^3 294 -> 275 us (272 before the
+// injected timeout, a choice of barrier per component).
 // ------------------------------------------------------------------------------------------------
 template <int N> struct SPlanOk {
   static constexpr bool ok = CPlan<N>::ok && CPlan<N>::NST == 2 && CPlan<N>::R(0) == CPlan<N>::T &&
