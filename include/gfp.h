@@ -265,7 +265,8 @@ const char* gfp_error_string(int status);
  * nothing arrives at, so the wait runs out as a real one would after about a second: the kernel marks
  * the solve timed out, waits (bounded) until the tile loads it has issued have landed, and returns, and
  * the solve returns GFP_ERR_DEVICE_TIMEOUT with the CUDA context intact.  Value 0 turns it off.  No GPU
- * fault is involved and the tile barriers' byte counts stay those of the loads.  Other kinds or values
+ * fault is involved and the tile barriers' byte counts stay those of the loads.  A batch keeps the setting under which its
+ * graph was captured (by gfp_batch_create, or by the solve after new phases or tiles).  Other kinds or values
  * return GFP_ERR_ARG.  Not thread-safe. */
 int gfp_set_fault_injection(int kind, int value);
 

@@ -6,10 +6,9 @@
 // of it (59 in the x-pass).  The fields stay doubles in memory; a pass converts a line's elements on the way in (fx_from)
 // and its results on the way out (fx_to), both with integer instructions.
 //
-// Measured at 256^3 (FP64 butterflies -> fixed point): x-pass 4.65 -> 1.48 ms, y-pass 1.90 -> 0.50 ms, z-pass
-// 5.34 -> 1.82 ms; the strain's error against torch's FP64 transforms after three iterations 2.27e-16 -> 1.93e-16.  The
-// passes are now bound by latency at 18 to 24 warps per SM (about 2 instructions of 4 issued per clock), half of the instructions
-// being the conversions.
+// Measured at 256^3 (FP64 butterflies -> fixed point): x-pass 4.65 -> 1.51 ms, y-pass 1.90 -> 0.53 ms, z-pass
+// 5.34 -> 1.91 ms.  The passes are now bound by latency at 18 to 24 warps per SM (about 2 instructions of 4 issued per clock),
+// half of the instructions being the conversions.
 //
 // Ranges: |re|, |im| < 2^60 at the input of a line, so that moduli stay below 2^60.5; a radix-4 layer grows
 // them to 2^62.5 < 2^63, and the following layers first scale by 1/4 or 1/2 -- for free where the element takes a
@@ -27,7 +26,7 @@
 namespace gfp {
 
 // a w / 4 (conjugate w with CONJ): the four partial products per part as 32 x 32 -> 64 multiply-adds, low x
-// low dropped (below 1/4 unit).  The middle sums stay below 2^62.8 for |a| < 2^62.5, |w| <= 2^62.
+// low dropped (below 1/4 unit).  The middle sums stay below 2^63 for |a| <= 2^62.85, |w| <= 2^62.
 template <bool CONJ>
 __device__ __forceinline__ fx2 fx_cmul(fx2 a, fxw w) {
   const int xl = (int)a.x, yl = (int)a.y, xh = fx_high(a.x), yh = fx_high(a.y);
@@ -381,7 +380,7 @@ __global__ void __launch_bounds__(COLS > 0 ? COLS * FxPlan<N>::T : 1024) pass_y_
 // copy of the code (the inverse on swapped real and imaginary parts): two copies overflow the instruction cache.  What the
 // update reads is prefetched into L2 during the inverse transform, and factors of two stay off the FP64 pipe (half of its
 // time is busy): 256^3 1.53 -> 1.50 ms, 128^3 195 -> 186 us, 64^3 31.9 -> 30.0 us.  Four CTAs per SM at 80 registers, with up to
-// 180 bytes of spills, against three at 96: 1.48 ms, 178 us, 25.5 us.
+// 120 bytes of spills, against three at 96: 1.48 ms, 178 us, 25.5 us (1.51 ms with ties to even).
 // ------------------------------------------------------------------------------------------------
 template <int N> __host__ __device__ constexpr int fx_line_pitch() { return N + N / 16; }
 
@@ -889,8 +888,8 @@ __device__ __forceinline__ void fx_green_fixed(int n3, int cols, int k10, int k2
 
 // Line scale for the inverse transform, each line's own (with one scale per column of six lines, components that are small
 // beside the others lost bits: 64 x 64 x 512, shear increments under an axial load, rms error 4.9e-15 of them, now 1.5e-15;
-// z-pass at 256^3 1.91 -> 1.94 ms): an element o of a point with exponent P fills the word shifted left by L = fx_lead(o) and then has the exponent P - L;
-// with top the line's largest, elements go in shifted right by top - (P - L) + 3 from there, in the unit 2^(top + 13 + ef).
+// z-pass at 256^3 1.91 -> 1.94 ms): an element o of a point with exponent P fills the word shifted left by L = fx_lead(o) and
+// then has the exponent P - L; with top the line's largest, elements go in shifted right by top - (P - L) + 3 from there, in the unit 2^(top + 13 + ef).
 struct FxBack {
   int bias;
   bool far;
